@@ -428,7 +428,7 @@ void build_hierarchy(Hier &H, cudaStream_t st)
         H.q32.alloc((size_t)n);
         H.z32.alloc((size_t)n);
     }
-    H.part.alloc(2 * (size_t)RED_MAX_BLOCKS);
+    H.part.alloc(4 * (size_t)RED_MAX_BLOCKS);  // two 16-byte records a block
     H.ctl.alloc(1);
     GW_CUDA(cudaMemsetAsync(H.ctl.p, 0, sizeof(Ctl), st));
     GW_CUDA(host_malloc((void **)&H.ctl_host, sizeof(Ctl)));

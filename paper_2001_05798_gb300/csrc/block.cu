@@ -342,6 +342,49 @@ __device__ __forceinline__ bool reduce_cols(const double (&loc)[NV][CW], double 
     return true;
 }
 
+// The same for FP32 pairs, in FP32 only (red_warp and its notes in kern.cuh):
+// a warp's NV * CW sums are handed over half by half, so a lane does 8
+// additions for 8 sums instead of 32, and no FP64 before the totals.
+template <int KB, int CW, int NV>
+__device__ __forceinline__ bool reduce_cols(const Sum2 (&loc)[NV][CW], double *part_, unsigned *cnt, double *tot)
+{
+    constexpr int TPR = KB / CW, W = BS / 32, N = NV * CW, NS = NV * KB;
+    static_assert(W == 8 && NS * W <= BS && NS * W % 32 == 0, "eight warps a block");
+    __shared__ Part sh[NS * W];
+    __shared__ unsigned ticket;
+    Part *part = reinterpret_cast<Part *>(part_);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    {
+        Sum2 a[N];
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+            for (int u = 0; u < CW; ++u) a[v * CW + u] = loc[v][u];
+        const Part p = red_pairs<N, TPR>(a, lane);
+        // one lane a sum writes: the lanes with zeros between the handed-over bits and TPR
+        if ((lane & (32 / N - 1) & ~(TPR - 1)) == 0) {
+            const int k = red_index<N>(lane);
+            sh[((k / CW) * KB + (lane % TPR) * CW + k % CW) * W + w] = p;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < NS * W) {
+        const Part p = red_eight(sh[threadIdx.x]);
+        if ((threadIdx.x & 7) == 0) part[(size_t)(threadIdx.x >> 3) * gridDim.x + blockIdx.x] = p;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) ticket = arrive_gpu(cnt);
+    __syncthreads();
+    if (ticket != gridDim.x - 1) return false;
+    for (int q = w; q < NS; q += W) {
+        const Part p = red_partials(part + (size_t)q * gridDim.x, (int)gridDim.x, lane, 32);
+        if (lane == 0) tot[q] = part_value(p);
+    }
+    if (threadIdx.x == 0) *cnt = 0u;
+    __syncthreads();
+    return true;
+}
+
 // after the column updates of an epilogue (thread 0 of the last block)
 template <int KB>
 __device__ __forceinline__ void refresh_done(BlkCtl *c)
@@ -368,7 +411,7 @@ __device__ __forceinline__ void col_stop(Ctl &c, int status)
 // Epilogue of the last kernel of a preconditioner application: rz = (r, z);
 // mode 1 also forms the flexible beta = -alpha (q, z) / rz_old.
 template <int KB, int CW>
-__device__ __forceinline__ void rz_cols(const double (&loc)[2][CW], double *part, BlkCtl *c, int mode)
+__device__ __forceinline__ void rz_cols(const Sum2 (&loc)[2][CW], double *part, BlkCtl *c, int mode)
 {
     __shared__ double tot[2 * KB];
     if (!reduce_cols<KB, CW, 2>(loc, part, &c->cnt[0], tot)) return;
@@ -389,25 +432,7 @@ __device__ __forceinline__ void rz_cols(const double (&loc)[2][CW], double *part
 }
 
 // A thread's per-column dot-product shares are error-free FP32 pairs carried
-// over all its rows (FP32 operations only) and become FP64 once, before the
-// block reduction, as in the single-vector passes.
-template <int NV, int CW>
-__device__ __forceinline__ void pairs_to_double(const Sum2 (&a)[NV][CW], double (&d)[NV][CW])
-{
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int u = 0; u < CW; ++u) d[v][u] = sum2_value(a[v][u]);
-}
-
-template <int KB, int CW>
-__device__ __forceinline__ void rz_cols(const Sum2 (&acc)[2][CW], double *part, BlkCtl *c, int mode)
-{
-    double loc[2][CW];
-    pairs_to_double(acc, loc);
-    rz_cols<KB, CW>(loc, part, c, mode);
-}
-
+// over all its rows, as in the single-vector passes.
 template <int CW>
 __device__ __forceinline__ void dot_cols(const float *b, const CV<float, CW> &z, const float *q, Sum2 (&loc)[2][CW])
 {
@@ -769,9 +794,7 @@ __global__ void __launch_bounds__(BS) kb_dir_spmv(M A, int n, const float *__res
 #pragma unroll
         for (int u = 0; u < CW; ++u) sum2_prod(acc[0][u], pi.v[u], qi.v[u]);
     }
-    double loc[1][CW];
-    pairs_to_double(acc, loc);
-    if (!reduce_cols<KB, CW, 1>(loc, part, &c->cnt[0], tot)) return;
+    if (!reduce_cols<KB, CW, 1>(acc, part, &c->cnt[0], tot)) return;
     if (threadIdx.x < KB) {
         Ctl &cj = c->col[threadIdx.x];
         if (!cj.done) {
@@ -819,9 +842,7 @@ __global__ void __launch_bounds__(BS) kb_update(int n, float *__restrict__ xs, f
         cst<CW>(xs + e, xv);
         cst<CW>(r + e, rv);
     }
-    double loc[1][CW];
-    pairs_to_double(acc, loc);
-    if (!reduce_cols<KB, CW, 1>(loc, part, &c->cnt[0], tot)) return;
+    if (!reduce_cols<KB, CW, 1>(acc, part, &c->cnt[0], tot)) return;
     if (threadIdx.x < KB) {
         Ctl &cj = c->col[threadIdx.x];
         if (!cj.done) {
@@ -1187,7 +1208,7 @@ static void ensure_state(Hier &H)
     s->p.alloc(m);
     s->pb.alloc(m);
     s->q.alloc(m);
-    s->part.alloc((size_t)2 * KB_MAX * RED_MAX_BLOCKS);
+    s->part.alloc((size_t)4 * KB_MAX * RED_MAX_BLOCKS);  // 2 KB_MAX 16-byte records a block
     s->ctl.alloc(1);
     GW_CUDA(cudaMemset(s->ctl.p, 0, sizeof(BlkCtl)));
     GW_CUDA(host_malloc((void **)&s->ctl_host, sizeof(BlkCtl)));

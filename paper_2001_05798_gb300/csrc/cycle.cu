@@ -687,11 +687,12 @@ static inline int vgrid(const Hier &, long long n) { return blocks_for(n); }
 // ------------------------------------------------------- V-cycle kernels --
 // Epilogue of the last kernel of a preconditioner application inside CG:
 // rz = (r, z); mode 1 also forms beta (flexible: -alpha (q,z) / rz_old).
-__device__ __forceinline__ void cg_rz_epilogue(VB vb, double lrz, double lqz, double *part, Ctl *c, int mode)
+template <class T>
+__device__ __forceinline__ void cg_rz_epilogue(VB vb, const DAcc (&acc)[2], double *part, Ctl *c, int mode)
 {
     if (!c) return;
-    double loc[2] = {lrz, lqz}, tot[2];
-    if (reduce_last<2>(vb, loc, part, &c->cnt[0], tot) && threadIdx.x == 0) {
+    double tot[2];
+    if (reduce_dots<T>(vb, acc, part, &c->cnt[0], tot)) {
         const double rz_new = tot[0];
         if (mode == 1) {
             const double beta = c->flexible ? -c->alpha * tot[1] / c->rz : rz_new / c->rz;
@@ -704,8 +705,7 @@ __device__ __forceinline__ void cg_rz_epilogue(VB vb, double lrz, double lqz, do
     }
 }
 
-// (b, z) and (q, z) contributions of R rows: products summed in T over the
-// R rows, then accumulated in FP64 across rows and threads
+// (b, z) and (q, z) contributions of R rows
 template <int R, class T, class OT>
 __device__ __forceinline__ void dot_rows(int i, const T *b, const OT (&z)[R], const T *q, DAcc &lrz, DAcc &lqz)
 {
@@ -765,7 +765,7 @@ __device__ __forceinline__ void b_jacobi(VB vb, M A, int n, const typename M::va
     using T = typename M::value_type;
     constexpr int R = M::R;
     if (finished(ctl)) return;
-    DAcc lrz, lqz;
+    DAcc acc[2];
     GROUP_ROWS(M, n)
     {
         VecN<T, R> ax;
@@ -784,10 +784,10 @@ __device__ __forceinline__ void b_jacobi(VB vb, M A, int n, const typename M::va
                 out[k] = (OT)xn;
             }
             st<R>(xo + i, o);
-            if constexpr (DOT) dot_rows<R>(i, b, out, q, lrz, lqz);
+            if constexpr (DOT) dot_rows<R>(i, b, out, q, acc[0], acc[1]);
         }
     }
-    if constexpr (DOT) cg_rz_epilogue(vb, dacc_value(lrz), dacc_value(lqz), part, ctl, mode);
+    if constexpr (DOT) cg_rz_epilogue<T>(vb, acc, part, ctl, mode);
 }
 
 template <class M, class BT, class OT, bool DOT>
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ void b_cheb0(VB vb, M A, int n, const typename M::val
     using T = typename M::value_type;
     constexpr int R = M::R;
     if (finished(ctl)) return;
-    DAcc lrz, lqz;
+    DAcc acc[2];
     GROUP_ROWS(M, n)
     {
         VecN<T, R> ax;
@@ -1175,13 +1175,13 @@ __device__ __forceinline__ void b_cheb0(VB vb, M A, int n, const typename M::val
                     out[k] = (OT)xn;
                 }
                 st<R>(xo + i, o);
-                dot_rows<R>(i, b, out, q, lrz, lqz);
+                dot_rows<R>(i, b, out, q, acc[0], acc[1]);
             } else {
                 if (x0zero) st<R>(x + i, dv);
             }
         }
     }
-    if constexpr (DOT) cg_rz_epilogue(vb, dacc_value(lrz), dacc_value(lqz), part, ctl, mode);
+    if constexpr (DOT) cg_rz_epilogue<T>(vb, acc, part, ctl, mode);
 }
 
 template <class M, class BT, class OT, bool DOT>
@@ -1211,7 +1211,7 @@ __device__ __forceinline__ void b_chebk(VB vb, M A, int n, const typename M::val
     using T = typename M::value_type;
     constexpr int R = M::R;
     if (finished(ctl)) return;
-    DAcc lrz, lqz;
+    DAcc acc[2];
     GROUP_ROWS(M, n)
     {
         const VecN<T, R> ad = A.dot(i, lane, GVec<T, T>{d});
@@ -1238,13 +1238,13 @@ __device__ __forceinline__ void b_chebk(VB vb, M A, int n, const typename M::val
                     out[k] = (OT)xn.v[k];
                 }
                 st<R>(xo + i, o);
-                dot_rows<R>(i, b0, out, q, lrz, lqz);
+                dot_rows<R>(i, b0, out, q, acc[0], acc[1]);
             } else {
                 st<R>(x + i, xn);
             }
         }
     }
-    if constexpr (DOT) cg_rz_epilogue(vb, dacc_value(lrz), dacc_value(lqz), part, ctl, mode);
+    if constexpr (DOT) cg_rz_epilogue<T>(vb, acc, part, ctl, mode);
 }
 
 template <class M, class OT, bool DOT>
@@ -1279,7 +1279,7 @@ __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M
     using T = typename M::value_type;
     constexpr int R = M::R;
     if (finished(ctl)) return;
-    DAcc lrz, lqz;
+    DAcc acc[2];
     GROUP_ROWS(M, n)
     {
         const VecN<T, R> ad = A.dot(i, lane, GProdC<T, T>{dw, b, c0});
@@ -1307,13 +1307,13 @@ __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M
                     out[k] = (OT)xv.v[k];
                 }
                 st<R>(xo + i, o);
-                dot_rows<R>(i, b, out, q, lrz, lqz);
+                dot_rows<R>(i, b, out, q, acc[0], acc[1]);
             } else {
                 st<R>(x + i, xv);
             }
         }
     }
-    if constexpr (DOT) cg_rz_epilogue(vb, dacc_value(lrz), dacc_value(lqz), part, ctl, mode);
+    if constexpr (DOT) cg_rz_epilogue<T>(vb, acc, part, ctl, mode);
 }
 
 template <class M, class OT, bool DOT>
@@ -1738,7 +1738,7 @@ __device__ __forceinline__ void b_cg_dir_spmv(VB vb, M A, int n, const typename 
         return;
     }
     const V beta = (V)c->beta;
-    DAcc acc;
+    DAcc acc[1];
     GROUP_ROWS(M, n)
     {
         const VecN<V, R> qi = A.dot(i, lane, GDir<V>{z, pold, beta});
@@ -1746,11 +1746,11 @@ __device__ __forceinline__ void b_cg_dir_spmv(VB vb, M A, int n, const typename 
             st<R>(q + i, qi);
             const VecN<V, R> pi = GDir<V>{z, pold, beta}.template vec<R>(i);
             st<R>(pnew + i, pi);
-            dot_add<R>(acc, pi.v, qi.v);
+            dot_add<R>(acc[0], pi.v, qi.v);
         }
     }
-    double loc[1] = {dacc_value(acc)}, tot[1];
-    if (reduce_last<1>(vb, loc, part, &c->cnt[0], tot) && threadIdx.x == 0) {
+    double tot[1];
+    if (reduce_dots<V>(vb, acc, part, &c->cnt[0], tot)) {
         const double pq = tot[0];
         c->pq = pq;
         c->it += 1;
@@ -1782,7 +1782,7 @@ __device__ __forceinline__ void b_cg_update(VB vb, int n, V *__restrict__ x, V *
     if (finished(c)) return;
     const V *__restrict__ p = (pb && !((c->it - 1) & 1)) ? pb : pa;
     const V a = (V)c->alpha;
-    DAcc acc;
+    DAcc acc[1];
     // two of the thread's row groups per step, all their loads issued first
     // (the second group's loads no longer wait for the first's); the groups
     // are added to the dot in the same order as one at a time
@@ -1804,7 +1804,7 @@ __device__ __forceinline__ void b_cg_update(VB vb, int n, V *__restrict__ x, V *
             xv.v[k] += a * pv.v[k];
             rv.v[k] -= a * qv.v[k];
         }
-        dot_add<R>(acc, rv.v, rv.v);
+        dot_add<R>(acc[0], rv.v, rv.v);
         st<R>(x + i, xv);
         st<R>(r + i, rv);
         if (two) {
@@ -1813,13 +1813,13 @@ __device__ __forceinline__ void b_cg_update(VB vb, int n, V *__restrict__ x, V *
                 xv2.v[k] += a * pv2.v[k];
                 rv2.v[k] -= a * qv2.v[k];
             }
-            dot_add<R>(acc, rv2.v, rv2.v);
+            dot_add<R>(acc[0], rv2.v, rv2.v);
             st<R>(x + i2, xv2);
             st<R>(r + i2, rv2);
         }
     }
-    double loc[1] = {dacc_value(acc)}, tot[1];
-    if (reduce_last<1>(vb, loc, part, &c->cnt[0], tot) && threadIdx.x == 0) {
+    double tot[1];
+    if (reduce_dots<V>(vb, acc, part, &c->cnt[0], tot)) {
         c->rr = tot[0];
         if (!isfinite(tot[0])) {
             ctl_stop(c, GW_ERR_BREAKDOWN);
