@@ -45,7 +45,7 @@ SINGLE_KERNELS = {
     "resid": "k_residual<MSten<float,4>,float> (stencil, b, x read, r written: 28 B/row)",
     "prolong": "k_prolong_imp<4> (s, fx, fy, fz, agg, x read, x written: 28 B/row + coarse vector)",
     "post1": "k_cheb0<MSten<float,4>,float,float,0> (stencil, dw, b, x read, r, d written: 36 B/row)",
-    "post2": "k_chebk<MSten<float,4>,float,1> (stencil, d, r, dw, x, b, q read, r, d2, z written: 52 B/row)",
+    "post2": "k_chebk<MSten<float,4>,float,1> (stencil, d, r, dw, x, b, q read, z written: 44 B/row)",
 }
 
 

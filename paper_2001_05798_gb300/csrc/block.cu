@@ -536,12 +536,13 @@ __global__ void __launch_bounds__(BS) kb_cheb0(M A, int n, const float *__restri
     if constexpr (DOT) rz_cols<KB, CW>(loc, part, c, mode);
 }
 
-// Chebyshev step k >= 2: r -= A d; dn = c1 d + c2 dw r; x += (add_prev ? d : 0) + dn
+// Chebyshev step k >= 2: r -= A d; dn = c1 d + c2 dw r; x += (add_prev ? d : 0) + dn;
+// the last step of an application (keep = 0, and DOT) stores neither r nor dn
 template <int KB, int CW, class M, bool DOT>
 __global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restrict__ dw, float *__restrict__ r,
                                                const float *__restrict__ d, float *__restrict__ dn, float *x,
                                                float *__restrict__ xo, float c1, float c2, int add_prev,
-                                               const float *__restrict__ b0, const float *__restrict__ q,
+                                               int keep, const float *__restrict__ b0, const float *__restrict__ q,
                                                double *part, BlkCtl *c, int mode)
 {
     pdl_enter();
@@ -560,8 +561,6 @@ __global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restri
             dv.v[u] = c1 * dp.v[u] + c2 * (w * ro.v[u]);
             xn.v[u] = xv.v[u] + (add_prev ? dp.v[u] : 0.f) + dv.v[u];
         }
-        cst<CW>(r + e, ro);
-        cst<CW>(dn + e, dv);
         if constexpr (DOT) {
             cst<CW>(xo + e, xn);
             dot_cols<CW>(b0 + e, xn, q ? q + e : nullptr, loc);
@@ -574,6 +573,10 @@ __global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restri
 
 // damped Jacobi: xo = x + dw (b - A x) (x = null: a zero guess)
 template <int KB, int CW, class M, bool DOT>
+            if (keep) {
+                cst<CW>(r + e, ro);
+                cst<CW>(dn + e, dv);
+            }
 __global__ void __launch_bounds__(BS) kb_jacobi(M A, int n, const float *__restrict__ dw, const float *__restrict__ b,
                                                 const float *__restrict__ x, float *__restrict__ xo,
                                                 const float *__restrict__ q, double *part, BlkCtl *c, int mode)
@@ -1047,11 +1050,11 @@ struct BCyc {
                         const bool f3 = fin && k == m - 1;
                         if (f3)
                             launch_pdl(kb_chebk<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
-                                       zout, (float)lv.c1[k], (float)lv.c2[k], 0, b, q, part, c, mode);
+                                       zout, (float)lv.c1[k], (float)lv.c2[k], 0, k < m - 1, b, q, part, c, mode);
                         else
                             launch_pdl(kb_chebk<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
-                                       (float *)nullptr, (float)lv.c1[k], (float)lv.c2[k], 0, (const float *)nullptr,
-                                       q, part, c, mode);
+                                       (float *)nullptr, (float)lv.c1[k], (float)lv.c2[k], 0, k < m - 1,
+                                       (const float *)nullptr, q, part, c, mode);
                         std::swap(d, dnx);
                     }
                     continue;
@@ -1067,10 +1070,10 @@ struct BCyc {
                     const int add_prev = (k == 1 && !zero) ? 1 : 0;
                     if (f2)
                         launch_pdl(kb_chebk<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p, zout,
-                                   (float)lv.c1[k], (float)lv.c2[k], add_prev, b, q, part, c, mode);
+                                   (float)lv.c1[k], (float)lv.c2[k], add_prev, k < m - 1, b, q, part, c, mode);
                     else
                         launch_pdl(kb_chebk<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
-                                   (float *)nullptr, (float)lv.c1[k], (float)lv.c2[k], add_prev,
+                                   (float *)nullptr, (float)lv.c1[k], (float)lv.c2[k], add_prev, k < m - 1,
                                    (const float *)nullptr, q, part, c, mode);
                     std::swap(d, dnx);
                 }

@@ -1197,14 +1197,17 @@ __global__ void __launch_bounds__(BS) k_cheb0(M A, int n, const typename M::valu
     b_cheb0<M, BT, OT, DOT>(vb_grid(), A, n, dw, b, x, r, d, xo, c0, x0zero, q, part, ctl, mode);
 }
 
-// Chebyshev step k >= 2: r -= A d; dn = c1 d + c2 dw r; x += (add_prev ? d : 0) + dn
+// Chebyshev step k >= 2: r -= A d; dn = c1 d + c2 dw r; x += (add_prev ? d : 0) + dn.
+// The pass is bound by its traffic: the last step of an application (keep = 0,
+// and every DOT pass) stores neither r nor dn, which nothing reads after it
+// (44 instead of 52 bytes a row of the FP32 level-0 pass with its dots).
 template <class M, class OT, bool DOT>
 __device__ __forceinline__ void b_chebk(VB vb, M A, int n, const typename M::value_type *__restrict__ dw,
                                               typename M::value_type *__restrict__ r,
                                               const typename M::value_type *__restrict__ d,
                                               typename M::value_type *__restrict__ dn, typename M::value_type *x,
                                               OT *__restrict__ xo, typename M::value_type c1,
-                                              typename M::value_type c2, int add_prev,
+                                              typename M::value_type c2, int add_prev, int keep,
                                               const typename M::value_type *__restrict__ b0,
                                               const typename M::value_type *__restrict__ q, double *part, Ctl *ctl,
                                               int mode) {
@@ -1227,8 +1230,6 @@ __device__ __forceinline__ void b_chebk(VB vb, M A, int n, const typename M::val
                 dv.v[k] = c1 * dp.v[k] + c2 * (w.v[k] * ro.v[k]);
                 xn.v[k] = xv.v[k] + (add_prev ? dp.v[k] : (T)0) + dv.v[k];
             }
-            st<R>(r + i, ro);
-            st<R>(dn + i, dv);
             if constexpr (DOT) {
                 OT out[R];
                 VecN<OT, R> o;
@@ -1253,19 +1254,23 @@ __global__ void __launch_bounds__(BS) k_chebk(M A, int n, const typename M::valu
                                               const typename M::value_type *__restrict__ d,
                                               typename M::value_type *__restrict__ dn, typename M::value_type *x,
                                               OT *__restrict__ xo, typename M::value_type c1,
-                                              typename M::value_type c2, int add_prev,
+                                              typename M::value_type c2, int add_prev, int keep,
                                               const typename M::value_type *__restrict__ b0,
                                               const typename M::value_type *__restrict__ q, double *part, Ctl *ctl,
                                               int mode)
 {
     pdl_enter();
-    b_chebk<M, OT, DOT>(vb_grid(), A, n, dw, r, d, dn, x, xo, c1, c2, add_prev, b0, q, part, ctl, mode);
+    b_chebk<M, OT, DOT>(vb_grid(), A, n, dw, r, d, dn, x, xo, c1, c2, add_prev, keep, b0, q, part, ctl, mode);
 }
 
 // The first two Chebyshev steps from a zero guess in one pass: with
 // d0 = c0 dw b (formed where gathered), r1 = b - A d0, d1 = c1 d0 + c2 dw r1,
 // x = d0 + d1.  r1 and d1 are stored only when more steps follow (keep).
 // DOT: x is the CG's z and (b, z), (q, z) are reduced.
+                if (keep) {
+                    st<R>(r + i, ro);
+                    st<R>(dn + i, dv);
+                }
 template <class M, class OT, bool DOT>
 __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M::value_type *__restrict__ dw,
                                                    const typename M::value_type *__restrict__ b,
@@ -1460,14 +1465,15 @@ static void smooth(Hier &H, std::vector<CycLevel<T>> &C, int l, const T *b, bool
                 for (int k = 2; k < m; ++k) {
                     const bool f3 = fin && k == m - 1;
                     timed(H, kind(), st, [&] {
-                        H.prof_bytes += vbytes(H, amat + dn * sx * 7.0 + (f3 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
+                        const int kp = k < m - 1;
+                        H.prof_bytes += vbytes(H, amat + dn * sx * (kp ? 7.0 : 5.0) + (f3 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
                         if (f3)
                             launch_pdl(k_chebk<M, T, true>, g, st, A, n, lv.dw.p, lv.r.p, d, dnx, lv.x.p, zout,
-                                       (T)lv.c1[k], (T)lv.c2[k], 0, b, q, part, ctl, mode);
+                                       (T)lv.c1[k], (T)lv.c2[k], 0, kp, b, q, part, ctl, mode);
                         else
                             launch_pdl(k_chebk<M, T, false>, g, st, A, n, lv.dw.p, lv.r.p, d, dnx, lv.x.p,
-                                       (T *)nullptr, (T)lv.c1[k], (T)lv.c2[k], 0, (const T *)nullptr, q, part, ctl,
-                                       mode);
+                                       (T *)nullptr, (T)lv.c1[k], (T)lv.c2[k], 0, kp, (const T *)nullptr, q, part,
+                                       ctl, mode);
                     });
                     std::swap(d, dnx);
                 }
@@ -1490,13 +1496,15 @@ static void smooth(Hier &H, std::vector<CycLevel<T>> &C, int l, const T *b, bool
                 const bool f2 = fin && k == m - 1;
                 const int add_prev = (k == 1 && !zero) ? 1 : 0;
                 timed(H, kind(), st, [&] {
-                    H.prof_bytes += vbytes(H, amat + dn * sx * 7.0 + (f2 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
+                    const int kp = k < m - 1;
+                    H.prof_bytes += vbytes(H, amat + dn * sx * (kp ? 7.0 : 5.0) + (f2 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
                     if (f2)
                         launch_pdl(k_chebk<M, T, true>, g, st, A, n, lv.dw.p, lv.r.p, d, dnx, lv.x.p, zout,
-                                   (T)lv.c1[k], (T)lv.c2[k], add_prev, b, q, part, ctl, mode);
+                                   (T)lv.c1[k], (T)lv.c2[k], add_prev, kp, b, q, part, ctl, mode);
                     else
                         launch_pdl(k_chebk<M, T, false>, g, st, A, n, lv.dw.p, lv.r.p, d, dnx, lv.x.p, (T *)nullptr,
-                                   (T)lv.c1[k], (T)lv.c2[k], add_prev, (const T *)nullptr, q, part, ctl, mode);
+                                   (T)lv.c1[k], (T)lv.c2[k], add_prev, kp, (const T *)nullptr, q, part, ctl,
+                                   mode);
                 });
                 std::swap(d, dnx);
             }
@@ -2357,8 +2365,9 @@ struct BSlot {
     Ctl *ctl;
 };
 
-// one launch of the batched iteration: pass kind, level, Chebyshev step and
-// whether the step reads d2 and writes d (the two direction buffers alternate)
+// one launch of the batched iteration: pass kind, level, Chebyshev step,
+// whether the step reads d2 and writes d (the two direction buffers alternate),
+// and whether its r and d are stored for a following step
 enum {
     BP_DIR_SPMV = 0, BP_UPDATE, BP_REL_FOLD, BP_REL_RES, BP_ZERO2, BP_CHEBK, BP_RESID, BP_RESTRICT_U,
     BP_RESTRICT_SUM, BP_SPMV, BP_COARSE, BP_PROLONG, BP_PROLONG_IMP, BP_CHEB0, BP_CHEBK_DOT
@@ -2433,11 +2442,11 @@ __global__ void __launch_bounds__(BS) kb_pass(const BSlot *__restrict__ slots, c
                 using M = decltype(A);
                 if constexpr (KIND == BP_CHEBK_DOT)
                     b_chebk<M, float, true>(vb, A, v.n, v.dw, v.r, d, dn, v.x, S.z32, v.c1[Lc.step], v.c2[Lc.step],
-                                            Lc.add_prev, (const float *)S.r32, S.q32, S.part, S.ctl, 1);
+                                            Lc.add_prev, 0, (const float *)S.r32, S.q32, S.part, S.ctl, 1);
                 else
                     b_chebk<M, float, false>(vb, A, v.n, v.dw, v.r, d, dn, v.x, (float *)nullptr, v.c1[Lc.step],
-                                             v.c2[Lc.step], Lc.add_prev, (const float *)nullptr, S.q32, S.part,
-                                             S.ctl, 1);
+                                             v.c2[Lc.step], Lc.add_prev, Lc.keep, (const float *)nullptr, S.q32,
+                                             S.part, S.ctl, 1);
             });
         } else if constexpr (KIND == BP_CHEB0) {
             const BLev &v = S.lv[l];
@@ -2608,7 +2617,7 @@ static std::vector<BLaunch> batch_sequence(int lmax, int m)
     for (int l = 0; l < lmax; ++l) {
         if (l < lmax - 1) {
             add(BP_ZERO2, l, 1, 0, 0, m > 2);
-            for (int k = 2; k < m; ++k) add(BP_CHEBK, l, k, (k % 2) ? 1 : 0, 0);  // k = 2 reads d, writes d2
+            for (int k = 2; k < m; ++k) add(BP_CHEBK, l, k, (k % 2) ? 1 : 0, 0, k < m - 1);  // k = 2 reads d, writes d2
             add(BP_RESID, l);
             if (l == 0) {
                 add(BP_RESTRICT_U, 0);
@@ -2623,7 +2632,7 @@ static std::vector<BLaunch> batch_sequence(int lmax, int m)
         add(l == 0 ? BP_PROLONG_IMP : BP_PROLONG, l);
         add(BP_CHEB0, l);
         for (int k = 1; k < m; ++k)
-            add(l == 0 && k == m - 1 ? BP_CHEBK_DOT : BP_CHEBK, l, k, (k % 2) ? 0 : 1, k == 1 ? 1 : 0);
+            add(l == 0 && k == m - 1 ? BP_CHEBK_DOT : BP_CHEBK, l, k, (k % 2) ? 0 : 1, k == 1 ? 1 : 0, k < m - 1);
     }
     return q;
 }
