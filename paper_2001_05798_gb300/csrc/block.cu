@@ -565,6 +565,10 @@ __global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restri
             cst<CW>(xo + e, xn);
             dot_cols<CW>(b0 + e, xn, q ? q + e : nullptr, loc);
         } else {
+            if (keep) {
+                cst<CW>(r + e, ro);
+                cst<CW>(dn + e, dv);
+            }
             cst<CW>(x + e, xn);
         }
     }
@@ -573,10 +577,6 @@ __global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restri
 
 // damped Jacobi: xo = x + dw (b - A x) (x = null: a zero guess)
 template <int KB, int CW, class M, bool DOT>
-            if (keep) {
-                cst<CW>(r + e, ro);
-                cst<CW>(dn + e, dv);
-            }
 __global__ void __launch_bounds__(BS) kb_jacobi(M A, int n, const float *__restrict__ dw, const float *__restrict__ b,
                                                 const float *__restrict__ x, float *__restrict__ xo,
                                                 const float *__restrict__ q, double *part, BlkCtl *c, int mode)

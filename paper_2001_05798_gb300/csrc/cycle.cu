@@ -1241,6 +1241,10 @@ __device__ __forceinline__ void b_chebk(VB vb, M A, int n, const typename M::val
                 st<R>(xo + i, o);
                 dot_rows<R>(i, b0, out, q, acc[0], acc[1]);
             } else {
+                if (keep) {
+                    st<R>(r + i, ro);
+                    st<R>(dn + i, dv);
+                }
                 st<R>(x + i, xn);
             }
         }
@@ -1267,10 +1271,6 @@ __global__ void __launch_bounds__(BS) k_chebk(M A, int n, const typename M::valu
 // d0 = c0 dw b (formed where gathered), r1 = b - A d0, d1 = c1 d0 + c2 dw r1,
 // x = d0 + d1.  r1 and d1 are stored only when more steps follow (keep).
 // DOT: x is the CG's z and (b, z), (q, z) are reduced.
-                if (keep) {
-                    st<R>(r + i, ro);
-                    st<R>(dn + i, dv);
-                }
 template <class M, class OT, bool DOT>
 __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M::value_type *__restrict__ dw,
                                                    const typename M::value_type *__restrict__ b,
