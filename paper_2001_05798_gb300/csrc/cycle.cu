@@ -830,28 +830,52 @@ __global__ void __launch_bounds__(BS) k_residual(M A, int n, const BT *__restric
     b_residual<M, BT>(vb_grid(), A, n, b, x, r, ctl);
 }
 
+// FP64 form: the first Chebyshev correction of the level that a restriction
+// writes to, d0 = c0 dw b, stored beside b (d0 null: not needed).  FP64 issue
+// bounds that level's pre-smoothing, and forming d0 from dw and b at every
+// entry cost two FP64 multiplications (and a gather) more an entry: at 96^3 the
+// level-1 pass took 44 us, 22 with the stored d0.  The FP32 form keeps forming it
+// where gathered: its level-1 pass is bound by fetching the matrix (15.9 against
+// 15.0 us at 128^3, and the restriction paid 1 us for the store).
+template <class T>
+struct First {
+    const T *__restrict__ dw;
+    T *__restrict__ d0;
+    T c0;
+    __device__ __forceinline__ void put(int i, T b) const
+    {
+        if constexpr (sizeof(T) == 8)
+            if (d0) d0[i] = c0 * (__ldg(dw + i) * b);
+    }
+};
+
 // y = R x (restriction)
 template <class M>
 __device__ __forceinline__ void b_spmv(VB vb, M Rm, int n, const typename M::value_type *__restrict__ x,
-                                             typename M::value_type *__restrict__ y, const Ctl *ctl) {
+                                       typename M::value_type *__restrict__ y,
+                                       const First<typename M::value_type> &f, const Ctl *ctl)
+{
     using T = typename M::value_type;
+    static_assert(M::R == 1, "restrictions are stored by rows");
     if (finished(ctl)) return;
     GROUP_ROWS(M, n)
     {
-        const VecN<T, M::R> s = Rm.dot(i, lane, GVec<T, T>{x});
+        const VecN<T, 1> s = Rm.dot(i, lane, GVec<T, T>{x});
         if (i < n && lane == 0) {
-            if constexpr (M::R == 1) y[out_row(Rm, i)] = s.v[0];
-            else st<M::R>(y + i, s);
+            const int o = out_row(Rm, i);
+            y[o] = s.v[0];
+            f.put(o, s.v[0]);
         }
     }
 }
 
 template <class M>
 __global__ void __launch_bounds__(BS) k_spmv(M Rm, int n, const typename M::value_type *__restrict__ x,
-                                             typename M::value_type *__restrict__ y, const Ctl *ctl)
+                                             typename M::value_type *__restrict__ y,
+                                             First<typename M::value_type> f, const Ctl *ctl)
 {
     pdl_enter();
-    b_spmv<M>(vb_grid(), Rm, n, x, y, ctl);
+    b_spmv<M>(vb_grid(), Rm, n, x, y, f, ctl);
 }
 
 // x += P e (interpolate and correct)
@@ -1268,10 +1292,13 @@ __global__ void __launch_bounds__(BS) k_chebk(M A, int n, const typename M::valu
 }
 
 // The first two Chebyshev steps from a zero guess in one pass: with
-// d0 = c0 dw b (formed where gathered), r1 = b - A d0, d1 = c1 d0 + c2 dw r1,
-// x = d0 + d1.  r1 and d1 are stored only when more steps follow (keep).
-// DOT: x is the CG's z and (b, z), (q, z) are reduced.
-template <class M, class OT, bool DOT>
+// d0 = c0 dw b (read from d0 with PRE, else formed where gathered), r1 = b - A d0,
+// d1 = c1 d0 + c2 dw r1, x = d0 + d1.  r1 and d1 are stored only when more steps
+// follow (keep).  DOT: x is the CG's z and (b, z), (q, z) are reduced.
+// PRE in the FP64 form: the restriction stores d0 on the coarser levels, a pass
+// of its own (k_first) on level 0, where the pre-smoothing so went from 54 us to
+// 27 + 7 at 96^3.
+template <class M, class OT, bool DOT, bool PRE>
 __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M::value_type *__restrict__ dw,
                                                    const typename M::value_type *__restrict__ b,
                                                    typename M::value_type *__restrict__ x,
@@ -1279,6 +1306,7 @@ __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M
                                                    typename M::value_type *__restrict__ d, OT *__restrict__ xo,
                                                    typename M::value_type c0, typename M::value_type c1,
                                                    typename M::value_type c2, int keep,
+                                                   const typename M::value_type *__restrict__ d0v,
                                                    const typename M::value_type *__restrict__ q, double *part,
                                                    Ctl *ctl, int mode) {
     using T = typename M::value_type;
@@ -1287,14 +1315,17 @@ __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M
     DAcc acc[2];
     GROUP_ROWS(M, n)
     {
-        const VecN<T, R> ad = A.dot(i, lane, GProdC<T, T>{dw, b, c0});
+        VecN<T, R> ad;
+        if constexpr (PRE) ad = A.dot(i, lane, GVec<T, T>{d0v});
+        else ad = A.dot(i, lane, GProdC<T, T>{dw, b, c0});
         if (i < n && lane == 0) {
             const VecN<T, R> bi = ld_ro<R>(b + i);
             const VecN<T, R> w = ld_ro<R>(dw + i);
-            VecN<T, R> rv, dv, xv;
+            VecN<T, R> rv, dv, xv, di;
+            if constexpr (PRE) di = ld_ro<R>(d0v + i);
 #pragma unroll
             for (int k = 0; k < R; ++k) {
-                const T d0 = c0 * (w.v[k] * bi.v[k]);
+                const T d0 = PRE ? di.v[k] : c0 * (w.v[k] * bi.v[k]);
                 rv.v[k] = bi.v[k] - ad.v[k];
                 dv.v[k] = c1 * d0 + c2 * (w.v[k] * rv.v[k]);
                 xv.v[k] = d0 + dv.v[k];
@@ -1321,7 +1352,7 @@ __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M
     if constexpr (DOT) cg_rz_epilogue<T>(vb, acc, part, ctl, mode);
 }
 
-template <class M, class OT, bool DOT>
+template <class M, class OT, bool DOT, bool PRE>
 __global__ void __launch_bounds__(BS) k_cheb_zero2(M A, int n, const typename M::value_type *__restrict__ dw,
                                                    const typename M::value_type *__restrict__ b,
                                                    typename M::value_type *__restrict__ x,
@@ -1329,11 +1360,23 @@ __global__ void __launch_bounds__(BS) k_cheb_zero2(M A, int n, const typename M:
                                                    typename M::value_type *__restrict__ d, OT *__restrict__ xo,
                                                    typename M::value_type c0, typename M::value_type c1,
                                                    typename M::value_type c2, int keep,
+                                                   const typename M::value_type *__restrict__ d0v,
                                                    const typename M::value_type *__restrict__ q, double *part,
                                                    Ctl *ctl, int mode)
 {
     pdl_enter();
-    b_cheb_zero2<M, OT, DOT>(vb_grid(), A, n, dw, b, x, r, d, xo, c0, c1, c2, keep, q, part, ctl, mode);
+    b_cheb_zero2<M, OT, DOT, PRE>(vb_grid(), A, n, dw, b, x, r, d, xo, c0, c1, c2, keep, d0v, q, part, ctl, mode);
+}
+
+// d0 = c0 dw b
+template <class T, int R>
+__global__ void __launch_bounds__(BS) k_first(int n, const T *__restrict__ dw, const T *__restrict__ b,
+                                              T *__restrict__ d0, T c0, const Ctl *ctl)
+{
+    pdl_enter();
+    if (finished(ctl)) return;
+    for (int i = R * (blockIdx.x * BS + threadIdx.x); i < n; i += R * gridDim.x * BS)
+        st<R>(d0 + i, GProdC<T, T>{dw, b, c0}.template vec<R>(i));
 }
 
 template <class T>
@@ -1455,12 +1498,19 @@ static void smooth(Hier &H, std::vector<CycLevel<T>> &C, int l, const T *b, bool
                 timed(H, kind(), st, [&] {
                     H.prof_bytes += vbytes(H, amat + 2.0 * dn * sx + (keep ? 3.0 : 1.0) * dn * sx +
                                                   (f2 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
-                    if (f2)
-                        launch_pdl(k_cheb_zero2<M, T, true>, g, st, A, n, lv.dw.p, b, lv.x.p, lv.r.p, d, zout,
-                                   (T)lv.c0, (T)lv.c1[1], (T)lv.c2[1], keep, q, part, ctl, mode);
-                    else
-                        launch_pdl(k_cheb_zero2<M, T, false>, g, st, A, n, lv.dw.p, b, lv.x.p, lv.r.p, d,
-                                   (T *)nullptr, (T)lv.c0, (T)lv.c1[1], (T)lv.c2[1], keep, q, part, ctl, mode);
+                    // d0 in d2, stored by the restriction on the coarser levels
+                    constexpr bool PRE = sizeof(T) == 8;
+                    const T *d0 = PRE ? lv.d2.p : nullptr;
+                    if (PRE && l == 0) {
+                        if (n % 2 == 0) launch_pdl(k_first<T, 2>, vgrid(H, n / 2), st, n, lv.dw.p, b, lv.d2.p, (T)lv.c0, ctl);
+                        else launch_pdl(k_first<T, 1>, vgrid(H, n), st, n, lv.dw.p, b, lv.d2.p, (T)lv.c0, ctl);
+                    }
+                    auto go = [&](auto kern, T *zo) {
+                        launch_pdl(kern, g, st, A, n, lv.dw.p, b, lv.x.p, lv.r.p, d, zo, (T)lv.c0, (T)lv.c1[1],
+                                   (T)lv.c2[1], keep, d0, q, part, ctl, mode);
+                    };
+                    if (f2) go(k_cheb_zero2<M, T, true, PRE>, zout);
+                    else go(k_cheb_zero2<M, T, false, PRE>, (T *)nullptr);
                 });
                 for (int k = 2; k < m; ++k) {
                     const bool f3 = fin && k == m - 1;
@@ -1548,20 +1598,24 @@ static void vcycle_t(Hier &H, std::vector<CycLevel<T>> &C, const T *r, T *z, Ctl
                 });
             });
         }
+        CycLevel<T> &lc = C[l + 1];
+        const bool cheb2 = H.o.smoother == GW_SMOOTH_CHEBYSHEV && H.o.degree >= 2;
+        const First<T> first{lc.dw.p, l + 1 < L - 1 && cheb2 ? lc.d2.p : nullptr, (T)lc.c0};
         timed(H, l0 ? GW_PK_RESTRICT : -1, st, [&] {
             if constexpr (sizeof(T) == 4) {
                 if (l0 && H.p0.n) {
                     // u pass: r, s, fx, fy, fz read, u written; sum pass: mem and u read,
                     // mptr read and r_c written per aggregate
                     H.prof_bytes += vbytes(H, 24.0 * dn + 8.0 * dn + 8.0 * (double)H.p0.nc);
-                    restrict_imp(H, lv.r.p, lv.t.p, C[1].b.p, ctl, st);
+                    restrict_imp(H, lv.r.p, lv.t.p, lc.b.p, ctl, st);
                     return;
                 }
             }
             H.prof_bytes += vbytes(H, mat_bytes(lv.R) + dn * sx + (double)lv.R.nr * sx);
             with_mat(lv.R, [&](auto Rm) {
                 using M = decltype(Rm);
-                launch_pdl(k_spmv<M>, grid_for<M>(H, lv.R.nr), st, Rm, lv.R.nr, lv.r.p, C[l + 1].b.p, ctl);
+                if constexpr (M::R == 1)
+                    launch_pdl(k_spmv<M>, grid_for<M>(H, lv.R.nr), st, Rm, lv.R.nr, lv.r.p, lc.b.p, first, ctl);
             });
         });
         GW_LAUNCH_CHECK();
@@ -2432,8 +2486,9 @@ __global__ void __launch_bounds__(BS) kb_pass(const BSlot *__restrict__ slots, c
             const float *bl = l == 0 ? S.r32 : v.b;
             with_bmat(v.A, [&](auto A) {
                 using M = decltype(A);
-                b_cheb_zero2<M, float, false>(vb, A, v.n, v.dw, bl, v.x, v.r, v.d, (float *)nullptr, v.c0, v.c1[1],
-                                              v.c2[1], Lc.keep, S.q32, S.part, S.ctl, 1);
+                b_cheb_zero2<M, float, false, false>(vb, A, v.n, v.dw, bl, v.x, v.r, v.d, (float *)nullptr, v.c0,
+                                                     v.c1[1], v.c2[1], Lc.keep, (const float *)nullptr, S.q32, S.part,
+                                                     S.ctl, 1);
             });
         } else if constexpr (KIND == BP_CHEBK || KIND == BP_CHEBK_DOT) {
             const BLev &v = S.lv[l];
@@ -2467,7 +2522,10 @@ __global__ void __launch_bounds__(BS) kb_pass(const BSlot *__restrict__ slots, c
             b_restrict_sum(vb, S.nc0, S.mptr, S.mem, S.lv[0].t, S.lv[1].b, S.ctl);
         } else if constexpr (KIND == BP_SPMV) {
             const BLev &v = S.lv[l];
-            with_bmat(v.R, [&](auto R) { b_spmv(vb, R, v.R.nr, (const float *)v.r, S.lv[l + 1].b, S.ctl); });
+            with_bmat(v.R, [&](auto R) {
+                using M = decltype(R);
+                if constexpr (M::R == 1) b_spmv(vb, R, v.R.nr, (const float *)v.r, S.lv[l + 1].b, First<float>{}, S.ctl);
+            });
         } else if constexpr (KIND == BP_COARSE) {
             const BLev &v = S.lv[l];
             b_coarse<float>(vb, v.n, S.Ainv, v.b, v.x, S.ctl);
