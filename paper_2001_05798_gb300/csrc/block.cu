@@ -105,8 +105,14 @@ struct BDir {
 // Row products of CW columns.  Terms are added in the order of the
 // single-vector views (stencil: -z, -y, -x, diagonal, +x, +y, +z; sliced
 // ELL: slot order), so a column's product equals the single-vector one.
+// WARP: a warp shares a row (the long rows of small levels), lanes of the same
+// columns taking every (32 / lanes of a row)-th entry and adding their sums by
+// shuffles.  With a thread a row and column group the 6438 rows of the third
+// level at 128^3 filled 50 blocks and each thread walked its row alone: a
+// restriction took 70 us, the smoothing passes 17-24 us.
 template <class T>
 struct BSten {
+    static constexpr bool WARP = false;
     const T *__restrict__ d;
     const T *__restrict__ ox;
     const T *__restrict__ oy;
@@ -131,6 +137,7 @@ struct BSten {
 
 template <class T>
 struct BSell {
+    static constexpr bool WARP = false;
     const int *__restrict__ sp;
     const int *__restrict__ ci;
     const T *__restrict__ v;
@@ -179,22 +186,31 @@ struct BSell {
 
 template <class T>
 struct BCsr {
+    static constexpr bool WARP = true;
     const int *__restrict__ rp;
     const int *__restrict__ ci;
     const T *__restrict__ v;
-    template <int CW, class F>
-    __device__ __forceinline__ CV<T, CW> dot(int i, F f) const
+    // el: this lane's place among the 32 / TPR lanes of its columns; every lane of
+    // the warp calls it and gets its columns' sums
+    template <int CW, int TPR, class F>
+    __device__ __forceinline__ CV<T, CW> dot_warp(int i, int el, F f) const
     {
         CV<T, CW> acc;
 #pragma unroll
         for (int u = 0; u < CW; ++u) acc.v[u] = 0;
         const int e1 = rp[i + 1];
-        for (int e = rp[i]; e < e1; ++e) cacc(acc, __ldg(v + e), f(__ldg(ci + e)));
+#pragma unroll 2
+        for (int e = rp[i] + el; e < e1; e += 32 / TPR) cacc(acc, __ldg(v + e), f(__ldg(ci + e)));
+#pragma unroll
+        for (int o = 16; o >= TPR; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < CW; ++u) acc.v[u] += __shfl_xor_sync(0xffffffffu, acc.v[u], o);
         return acc;
     }
 };
 
 struct BStenB {
+    static constexpr bool WARP = false;
     const float *__restrict__ d;
     const __nv_bfloat16 *__restrict__ ox;
     const __nv_bfloat16 *__restrict__ oy;
@@ -218,6 +234,7 @@ struct BStenB {
 };
 
 struct BStenH {
+    static constexpr bool WARP = false;
     const float *__restrict__ sd;
     const __half *__restrict__ dd;
     const __half *__restrict__ ox;
@@ -280,6 +297,22 @@ static void with_bmat(const MatStore<T> &M, F f)
     default: fail(GW_ERR_ARG, "interleaved solves need P, R and the coarse operators uncompressed");
     }
 }
+
+// the row product of a thread's columns (lane el of a WARP view)
+template <int CW, int TPR, class M, class F>
+__device__ __forceinline__ auto bdot(const M &A, int i, int el, F f)
+{
+    if constexpr (M::WARP) return A.template dot_warp<CW, TPR>(i, el, f);
+    else return A.template dot<CW>(i, f);
+}
+
+// thread -> (row, first column, lane el among those of the same columns):
+// TPR = KB / CW threads per row, or a warp per row of a WARP view
+#define MAT_ROWS(M, n, KB, CW)                                                                          \
+    constexpr int TPR_ = (KB) / (CW), LPR_ = M::WARP ? 32 : TPR_;                                       \
+    for (int t_ = blockIdx.x * BS + threadIdx.x, i = t_ / LPR_, off = (t_ % TPR_) * (CW),                \
+             el = (t_ % LPR_) / TPR_;                                                                   \
+         i < (n); t_ += gridDim.x * BS, i = t_ / LPR_)
 
 // thread -> (row, first column): TPR = KB / CW threads per row
 #define BLOCK_ROWS(n, KB, CW)                                                                         \
@@ -462,9 +495,10 @@ __global__ void __launch_bounds__(BS) kb_cheb_zero2(M A, int n, const float *__r
     pdl_enter();
     if (bfinished(c)) return;
     Sum2 loc[2][CW];
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
-        const CV<float, CW> ad = A.template dot<CW>(i, BProd<CW, KB>{dw, b + off, c0});
+        const CV<float, CW> ad = bdot<CW, TPR_>(A, i, el, BProd<CW, KB>{dw, b + off, c0});
+        if (M::WARP && el) continue;
         const size_t e = (size_t)i * KB + off;
         const CV<float, CW> bi = cld<CW>(b + e);
         const float w = dw[i];
@@ -501,12 +535,13 @@ __global__ void __launch_bounds__(BS) kb_cheb0(M A, int n, const float *__restri
     pdl_enter();
     if (bfinished(c)) return;
     Sum2 loc[2][CW];
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
         CV<float, CW> ax;
 #pragma unroll
         for (int u = 0; u < CW; ++u) ax.v[u] = 0.f;
-        if (!x0zero) ax = A.template dot<CW>(i, BVec<float, CW, KB>{x + off});
+        if (!x0zero) ax = bdot<CW, TPR_>(A, i, el, BVec<float, CW, KB>{x + off});
+        if (M::WARP && el) continue;
         const size_t e = (size_t)i * KB + off;
         const CV<float, CW> bi = cld<CW>(b + e);
         const float w = dw[i];
@@ -548,9 +583,10 @@ __global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restri
     pdl_enter();
     if (bfinished(c)) return;
     Sum2 loc[2][CW];
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
-        const CV<float, CW> ad = A.template dot<CW>(i, BVec<float, CW, KB>{d + off});
+        const CV<float, CW> ad = bdot<CW, TPR_>(A, i, el, BVec<float, CW, KB>{d + off});
+        if (M::WARP && el) continue;
         const size_t e = (size_t)i * KB + off;
         const CV<float, CW> rv = cld<CW>(r + e), dp = cld<CW>(d + e), xv = cld<CW>(x + e);
         const float w = dw[i];
@@ -584,16 +620,17 @@ __global__ void __launch_bounds__(BS) kb_jacobi(M A, int n, const float *__restr
     pdl_enter();
     if (bfinished(c)) return;
     Sum2 loc[2][CW];
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
         CV<float, CW> ax, xv;
 #pragma unroll
         for (int u = 0; u < CW; ++u) ax.v[u] = xv.v[u] = 0.f;
         const size_t e = (size_t)i * KB + off;
         if (x) {
-            ax = A.template dot<CW>(i, BVec<float, CW, KB>{x + off});
+            ax = bdot<CW, TPR_>(A, i, el, BVec<float, CW, KB>{x + off});
             xv = cld<CW>(x + e);
         }
+        if (M::WARP && el) continue;
         const CV<float, CW> bi = cld<CW>(b + e);
         const float w = dw[i];
         CV<float, CW> xn;
@@ -621,9 +658,10 @@ __global__ void __launch_bounds__(BS) kb_residual(M A, int n, const float *__res
 {
     pdl_enter();
     if (bfinished(c)) return;
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
-        const CV<float, CW> ax = A.template dot<CW>(i, BVec<float, CW, KB>{x + off});
+        const CV<float, CW> ax = bdot<CW, TPR_>(A, i, el, BVec<float, CW, KB>{x + off});
+        if (M::WARP && el) continue;
         const size_t e = (size_t)i * KB + off;
         CV<float, CW> ro = cld<CW>(b + e);
 #pragma unroll
@@ -639,9 +677,10 @@ __global__ void __launch_bounds__(BS) kb_spmv(M Rm, int n, const float *__restri
 {
     pdl_enter();
     if (bfinished(c)) return;
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
-        const CV<float, CW> s = Rm.template dot<CW>(i, BVec<float, CW, KB>{x + off});
+        const CV<float, CW> s = bdot<CW, TPR_>(Rm, i, el, BVec<float, CW, KB>{x + off});
+        if (M::WARP && el) continue;
         int o = i;
         if constexpr (std::is_same<M, BSell<float>>::value) o = Rm.out_row(i);
         cst<CW>(y + (size_t)o * KB + off, s);
@@ -655,9 +694,10 @@ __global__ void __launch_bounds__(BS) kb_prolong(M P, int n, const float *__rest
 {
     pdl_enter();
     if (bfinished(c)) return;
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
-        const CV<float, CW> s = P.template dot<CW>(i, BVec<float, CW, KB>{ec + off});
+        const CV<float, CW> s = bdot<CW, TPR_>(P, i, el, BVec<float, CW, KB>{ec + off});
+        if (M::WARP && el) continue;
         const size_t e = (size_t)i * KB + off;
         CV<float, CW> xv = cld<CW>(x + e);
 #pragma unroll
@@ -786,10 +826,11 @@ __global__ void __launch_bounds__(BS) kb_dir_spmv(M A, int n, const float *__res
     CV<float, CW> beta;  // a thread keeps its columns: the grid stride is a multiple of KB / CW
 #pragma unroll
     for (int u = 0; u < CW; ++u) beta.v[u] = (float)c->col[first_col<KB, CW>() + u].beta;
-    BLOCK_ROWS(n, KB, CW)
+    MAT_ROWS(M, n, KB, CW)
     {
         const BDir<CW, KB> f{z + off, pold + off, beta};
-        const CV<float, CW> qi = A.template dot<CW>(i, f);
+        const CV<float, CW> qi = bdot<CW, TPR_>(A, i, el, f);
+        if (M::WARP && el) continue;
         const CV<float, CW> pi = f(i);
         const size_t e = (size_t)i * KB + off;
         cst<CW>(q + e, qi);
@@ -893,10 +934,12 @@ __global__ void __launch_bounds__(BS) kb_rel_res(M A, int n, const double *__res
         mine[u] = !force && c->col[first_col<KB, CW>() + u].check != 0;
         act |= mine[u];
     }
-    BLOCK_ROWS(n, KB, CW)
+    if constexpr (M::WARP) act = __any_sync(0xffffffffu, act);
+    MAT_ROWS(M, n, KB, CW)
     {
         if (!act) break;
-        const CV<double, CW> ax = A.template dot<CW>(i, BVec<double, CW, KB>{x + off});
+        const CV<double, CW> ax = bdot<CW, TPR_>(A, i, el, BVec<double, CW, KB>{x + off});
+        if (M::WARP && el) continue;
         const size_t e = (size_t)i * KB + off;
         const CV<double, CW> bv = cld<CW>(b + e);
 #pragma unroll
@@ -1000,6 +1043,11 @@ struct BCyc {
     cudaStream_t st;
 
     int g(int n) const { return bgrid(H, (long long)n * TPR); }
+    template <class M>
+    int gm(int n) const
+    {
+        return bgrid(H, (long long)n * (M::WARP ? 32 : TPR));
+    }
 
     // one smoothing application on level l (the single-vector smoother's steps)
     void smooth(int l, const float *b, bool x0zero, bool last, float *zout, const float *q, int mode)
@@ -1015,9 +1063,9 @@ struct BCyc {
                     const bool first = x0zero && s == 0, fin = last && s == nu - 1;
                     const float *xi = first ? nullptr : cur;
                     if (fin)
-                        launch_pdl(kb_jacobi<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, b, xi, zout, q, part, c, mode);
+                        launch_pdl(kb_jacobi<KB, CW, M, true>, gm<M>(n), st, A, n, lv.dw.p, b, xi, zout, q, part, c, mode);
                     else
-                        launch_pdl(kb_jacobi<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, b, xi, nxt, q, part, c,
+                        launch_pdl(kb_jacobi<KB, CW, M, false>, gm<M>(n), st, A, n, lv.dw.p, b, xi, nxt, q, part, c,
                                    mode);
                     if (!fin) std::swap(cur, nxt);
                 }
@@ -1032,7 +1080,7 @@ struct BCyc {
                 const bool fin = last && s == nu - 1;
                 float *d = bl.d.p, *dnx = bl.d2.p;
                 if (fin && m == 1) {
-                    launch_pdl(kb_cheb0<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d, zout,
+                    launch_pdl(kb_cheb0<KB, CW, M, true>, gm<M>(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d, zout,
                                (float)lv.c0, zero, q, part, c, mode);
                     continue;
                 }
@@ -1040,26 +1088,26 @@ struct BCyc {
                     const bool f2 = fin && m == 2;
                     const int keep = m > 2;
                     if (f2)
-                        launch_pdl(kb_cheb_zero2<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d,
+                        launch_pdl(kb_cheb_zero2<KB, CW, M, true>, gm<M>(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d,
                                    zout, (float)lv.c0, (float)lv.c1[1], (float)lv.c2[1], keep, q, part, c, mode);
                     else
-                        launch_pdl(kb_cheb_zero2<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d,
+                        launch_pdl(kb_cheb_zero2<KB, CW, M, false>, gm<M>(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d,
                                    (float *)nullptr, (float)lv.c0, (float)lv.c1[1], (float)lv.c2[1], keep, q, part, c,
                                    mode);
                     for (int k = 2; k < m; ++k) {
                         const bool f3 = fin && k == m - 1;
                         if (f3)
-                            launch_pdl(kb_chebk<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
+                            launch_pdl(kb_chebk<KB, CW, M, true>, gm<M>(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
                                        zout, (float)lv.c1[k], (float)lv.c2[k], 0, k < m - 1, b, q, part, c, mode);
                         else
-                            launch_pdl(kb_chebk<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
+                            launch_pdl(kb_chebk<KB, CW, M, false>, gm<M>(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
                                        (float *)nullptr, (float)lv.c1[k], (float)lv.c2[k], 0, k < m - 1,
                                        (const float *)nullptr, q, part, c, mode);
                         std::swap(d, dnx);
                     }
                     continue;
                 }
-                launch_pdl(kb_cheb0<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d,
+                launch_pdl(kb_cheb0<KB, CW, M, false>, gm<M>(n), st, A, n, lv.dw.p, b, bl.x.p, bl.r.p, d,
                            (float *)nullptr, (float)lv.c0, zero, q, part, c, mode);
                 if (m == 1) {
                     if (!zero) launch_pdl(kb_axpy<KB>, bgrid(H, (long long)n * KB), st, (long long)n * KB, d, bl.x.p, c);
@@ -1069,10 +1117,10 @@ struct BCyc {
                     const bool f2 = fin && k == m - 1;
                     const int add_prev = (k == 1 && !zero) ? 1 : 0;
                     if (f2)
-                        launch_pdl(kb_chebk<KB, CW, M, true>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p, zout,
+                        launch_pdl(kb_chebk<KB, CW, M, true>, gm<M>(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p, zout,
                                    (float)lv.c1[k], (float)lv.c2[k], add_prev, k < m - 1, b, q, part, c, mode);
                     else
-                        launch_pdl(kb_chebk<KB, CW, M, false>, g(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
+                        launch_pdl(kb_chebk<KB, CW, M, false>, gm<M>(n), st, A, n, lv.dw.p, bl.r.p, d, dnx, bl.x.p,
                                    (float *)nullptr, (float)lv.c1[k], (float)lv.c2[k], add_prev, k < m - 1,
                                    (const float *)nullptr, q, part, c, mode);
                     std::swap(d, dnx);
@@ -1093,11 +1141,11 @@ struct BCyc {
             smooth(l, b, true, false, nullptr, q, mode);
             with_bmat(lv.A, [&](auto A) {
                 using M = decltype(A);
-                launch_pdl(kb_residual<KB, CW, M>, g(n), st, A, n, b, (const float *)bl.x.p, bl.r.p, (const BlkCtl *)c);
+                launch_pdl(kb_residual<KB, CW, M>, gm<M>(n), st, A, n, b, (const float *)bl.x.p, bl.r.p, (const BlkCtl *)c);
             });
             with_bmat(lv.R, [&](auto Rm) {
                 using M = decltype(Rm);
-                launch_pdl(kb_spmv<KB, CW, M>, g(lv.R.nr), st, Rm, lv.R.nr, (const float *)bl.r.p, S.lv[l + 1].b.p,
+                launch_pdl(kb_spmv<KB, CW, M>, gm<M>(lv.R.nr), st, Rm, lv.R.nr, (const float *)bl.r.p, S.lv[l + 1].b.p,
                            (const BlkCtl *)c);
             });
         }
@@ -1118,7 +1166,7 @@ struct BCyc {
             }
             with_bmat(lv.P, [&](auto P) {
                 using M = decltype(P);
-                launch_pdl(kb_prolong<KB, CW, M>, g(n), st, P, n, (const float *)S.lv[l + 1].x.p, bl.x.p,
+                launch_pdl(kb_prolong<KB, CW, M>, gm<M>(n), st, P, n, (const float *)S.lv[l + 1].x.p, bl.x.p,
                            (const BlkCtl *)c);
             });
             smooth(l, l == 0 ? r : bl.b.p, false, l == 0, z, q, mode);
@@ -1132,7 +1180,7 @@ struct BCyc {
         launch_pdl(kb_rel_fold<KB>, bgrid(H, (long long)n * KB), st, n, S.x64.p, S.xs.p, (const BlkCtl *)c, force);
         with_bmat(H.A64, [&](auto A) {
             using M = decltype(A);
-            launch_pdl(kb_rel_res<KB, 2, M>, bgrid(H, (long long)n * (KB / 2)), st, A, n, (const double *)S.b64.p,
+            launch_pdl(kb_rel_res<KB, 2, M>, bgrid(H, (long long)n * (M::WARP ? 32 : KB / 2)), st, A, n, (const double *)S.b64.p,
                        (const double *)S.x64.p, S.r.p, part, c, force);
         });
     }
@@ -1151,7 +1199,7 @@ struct BCyc {
         float *pold = parity ? S.pb.p : S.p.p, *pnew = parity ? S.p.p : S.pb.p;
         with_bmat(cg_op32(H), [&](auto A) {
             using M = decltype(A);
-            launch_pdl(kb_dir_spmv<KB, CW, M>, g(n), st, A, n, (const float *)S.z.p, (const float *)pold, pnew, S.q.p,
+            launch_pdl(kb_dir_spmv<KB, CW, M>, gm<M>(n), st, A, n, (const float *)S.z.p, (const float *)pold, pnew, S.q.p,
                        part, c);
         });
         launch_pdl(kb_update<KB, CW>, g(n), st, n, S.xs.p, S.r.p, (const float *)pnew, (const float *)S.q.p, part, c);
