@@ -2381,7 +2381,13 @@ int pcg_run(Hier &H, double tol, int maxit, int *iters, double *relres, cudaStre
 // independently: a finished slot's passes return at once until it is taken.
 
 constexpr int BATCH_MAXL = 12;   // levels of a hierarchy in a batch
-constexpr int BATCH_NB_CAP = 1024;  // virtual blocks of one pass of one slot
+// Virtual blocks of one pass of one slot.  A work item costs a few microseconds
+// whatever its rows (slot table, descriptor and first loads one after the other,
+// a reduction's barriers), so a slot has no more of them than two a SM.  Against
+// 1024 (ms a set of solves to 1e-12): eight of sides 33-96 18.6 -> 16.4, 45 and
+// 57 4.6 -> 3.9, one of 96 6.4 -> 6.0, four of 160 59.2 -> 56.1; 152 loses on few
+// larger solves (one of 96 7.5), 608 gains less.
+constexpr int BATCH_NB_CAP = 304;
 
 enum { BM_NONE = 0, BM_STEN4, BM_STEN2, BM_STEN1, BM_SELL, BM_CSR32 };
 
