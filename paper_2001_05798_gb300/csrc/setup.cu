@@ -30,11 +30,6 @@ static inline int nblk(long long n, int bs, long long cap = 152LL * 32)
 
 #define GRID_STRIDE(i, n) for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
 
-// Row-parallel form of the SpGEMM and prolongator passes: chosen per product
-// from the row counts and lengths (0), or forced to a thread a row (1) or a
-// warp a row (2) by GW_SETUP_FORMS=thread|warp in the environment, read once,
-// so that tests can check both forms against the oracle on any problem.  Both
-// forms give the same bits.
 // Lanes that share a row in the per-row setup passes: one for the short rows
 // of the fine grid, a group of 8 or a warp for the long rows of the coarse
 // levels (a thread walking a row of a hundred entries alone leaves a
@@ -52,6 +47,11 @@ static int row_lanes(const DCSR &A)
                    ii##_step = (long long)gridDim.x * (blockDim.x / (G));                        \
          (G) == 1 ? ii < (n) : __any_sync(0xffffffffu, ii < (n)); ii += ii##_step)
 
+// Row-parallel form of the SpGEMM and prolongator passes: chosen per product
+// from the row counts and lengths (0), or forced to a thread a row (SpGEMM: a
+// group of lanes a row) (1) or a warp a row (2) by GW_SETUP_FORMS=thread|warp in
+// the environment, read once, so that tests can check both forms against the
+// oracle on any problem.  Both forms give the same bits.
 static int setup_forms()
 {
     static const int f = [] {
@@ -1051,144 +1051,238 @@ __global__ void k_sg_numeric(int nr, const int *__restrict__ rows, const int *__
     }
 }
 
-// Short rows, one thread each: the distinct columns of the row kept as a
-// sorted list in shared memory (entry t of thread x at [t * SGT_BS + x], so
-// the threads of a warp touch distinct banks).  Symbolic: counts the row's
-// distinct columns; a row with more than SGT_CAP of them goes to the warp
-// kernels' row list instead.  Numeric: inserts each product L(i,k) Rm(k,c)
-// in L's column order k, so every output entry receives its terms in
-// ascending k, the same sums as the warp kernel forms.
-constexpr int SGT_BS = 128, SGT_CAP = 64;
-
-__device__ __forceinline__ int sgt_find(const int *list, int u, int c)
-{
-    int lo = 0, hi = u;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (list[mid * SGT_BS] < c) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-__global__ void __launch_bounds__(SGT_BS) k_sgt_symbolic(int nr, const int *__restrict__ lrp, const int *__restrict__ lci,
-                                                        const int *__restrict__ rrp, const int *__restrict__ rci,
-                                                        int *__restrict__ cnt, int *__restrict__ long_rows,
-                                                        int *__restrict__ nlong, int *__restrict__ maxu)
-{
-    __shared__ int sl[SGT_CAP * SGT_BS];
-    int *list = sl + threadIdx.x;
-    int best = 0;
-    GRID_STRIDE(ii, nr)
-    {
-        const int i = (int)ii;
-        int u = 0;
-        bool over = false;
-        for (int e = lrp[i]; e < lrp[i + 1] && !over; ++e) {
-            const int k = lci[e];
-            for (int f = rrp[k]; f < rrp[k + 1]; ++f) {
-                const int c = rci[f];
-                const int pos = sgt_find(list, u, c);
-                if (pos < u && list[pos * SGT_BS] == c) continue;
-                if (u == SGT_CAP) {
-                    over = true;
-                    break;
-                }
-                for (int t = u; t > pos; --t) list[t * SGT_BS] = list[(t - 1) * SGT_BS];
-                list[pos * SGT_BS] = c;
-                ++u;
-            }
-        }
-        if (over) {
-            long_rows[atomicAdd(nlong, 1)] = i;
-        } else {
-            cnt[i] = u;
-            best = max(best, u);
-        }
-    }
-    if (best > 0) atomicMax(maxu, best);
-}
+// A group of G lanes per row, in one pass over the products: the row's distinct
+// columns in an open-addressing table in shared memory (key, and the position
+// at which the column first came up), their sums by position.  The group walks
+// L's row in order and its lanes take the entries of Rm's row k, which have
+// distinct columns, so every output entry receives its terms in ascending k; the
+// columns are rank-sorted at the end and the row goes to a temporary of CAP
+// entries a row, packed once the row pointers are known (crp null); where that
+// temporary would be too large, a first run only counts (oci null) and a second,
+// with the row pointers crp, writes each row in its place.  A row of more than
+// CAP distinct columns goes to the warp kernels' row list (the second run leaves
+// it out).
+// What bounds the product is the chain of dependent loads per entry of L and
+// FP64 issue (a warp instruction holds the SM's FP64 units for 16 cycles however
+// few lanes work): with a warp a row, 4 of 32 lanes worked on A_1 P_1 and 8 on
+// R_0 (A P)_0, in two passes.  So G follows the mean row length of Rm, G entries
+// of L are loaded at once and SGG_PF of their rows before the first is added.
+// At 160^3 (us): A_0 P_0 1592 -> 1350 (against a thread a row with the row in
+// shared memory), R_0 (A P)_0 4740 -> 1350, A_1 P_1 2890 -> 840, R_1 (A P)_1
+// 1660 -> 450; at 45^3 the four together 700 -> 330.
+constexpr int SGG_BS = 128, SGG_PF = 4;
+#ifndef GW_SGG_TEMP_MAX
+#define GW_SGG_TEMP_MAX (4.0 * (1 << 30))
+#endif
+constexpr double SGG_TEMP_MAX = GW_SGG_TEMP_MAX;
 
 template <int CAP>
-__global__ void __launch_bounds__(SGT_BS) k_sgt_numeric(int nr, const int *__restrict__ lrp, const int *__restrict__ lci,
-                                                       const double *__restrict__ lv, const int *__restrict__ rrp,
-                                                       const int *__restrict__ rci, const double *__restrict__ rv,
-                                                       const int *__restrict__ crp, int *__restrict__ cci,
-                                                       double *__restrict__ cv)
+constexpr size_t sgg_group_bytes()
 {
-    extern __shared__ double sgt_smem[];  // acc[CAP * SGT_BS] doubles, then list[CAP * SGT_BS] ints
-    double *acc = sgt_smem + threadIdx.x;
-    int *list = (int *)(sgt_smem + CAP * SGT_BS) + threadIdx.x;
-    GRID_STRIDE(ii, nr)
-    {
-        const int i = (int)ii;
-        const int o = crp[i], cnt = crp[i + 1] - o;
-        if (cnt > CAP) continue;  // a long row: the warp kernel's
-        int u = 0;
-        for (int e = lrp[i]; e < lrp[i + 1]; ++e) {
-            const int k = lci[e];
-            const double a = lv[e];
-            for (int f = rrp[k]; f < rrp[k + 1]; ++f) {
-                const int c = rci[f];
-                const int pos = sgt_find(list, u, c);
-                if (!(pos < u && list[pos * SGT_BS] == c)) {
-                    for (int t = u; t > pos; --t) {
-                        list[t * SGT_BS] = list[(t - 1) * SGT_BS];
-                        acc[t * SGT_BS] = acc[(t - 1) * SGT_BS];
+    return (size_t)CAP * 8 + 2 * CAP * 4 + CAP * 4 + 2 * CAP;  // sums, keys, columns, positions
+}
+template <int G, int CAP>
+constexpr size_t sgg_smem()
+{
+    return (SGG_BS / G) * (sgg_group_bytes<CAP>() + sizeof(int));
+}
+
+// position of column c in the row's table (inserted if new; >= CAP: no room)
+template <int CAP>
+__device__ __forceinline__ int sgg_find(volatile int *keys, volatile unsigned char *pos, int *count, int *cols,
+                                        double *acc, int c)
+{
+    unsigned h = sg_hash(c) >> 8 & (unsigned)(2 * CAP - 1);
+    for (;;) {
+        const int k = keys[h];
+        if (k == c) return pos[h];
+        if (k == -1 && atomicCAS((int *)&keys[h], -1, c) == -1) {
+            const int p = atomicAdd(count, 1);
+            if (p < CAP) {
+                pos[h] = (unsigned char)p;
+                cols[p] = c;
+                acc[p] = 0.0;
+            }
+            return p;
+        }
+        h = (h + 1) & (unsigned)(2 * CAP - 1);
+    }
+}
+
+template <int G, int CAP>
+__global__ void __launch_bounds__(SGG_BS) k_sgg(int nr, const int *__restrict__ lrp, const int *__restrict__ lci,
+                                                const double *__restrict__ lv, const int *__restrict__ rrp,
+                                                const int *__restrict__ rci, const double *__restrict__ rv,
+                                                const int *__restrict__ crp, int *__restrict__ cnt,
+                                                int *__restrict__ oci, double *__restrict__ ov,
+                                                int *__restrict__ long_rows, int *__restrict__ nlong)
+{
+    // the step that passes CAP columns inserts at most G more keys and is the
+    // row's last, so the table never fills
+    static_assert(G >= SGG_PF && 2 * G <= CAP && CAP <= 256, "group and table sizes");
+    extern __shared__ double sgg_mem[];
+    constexpr int NG = SGG_BS / G;
+    const int g = threadIdx.x / G, lane = threadIdx.x & (G - 1);
+    const unsigned all = 0xffffffffu;
+    const unsigned mine = G == 32 ? all : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+    double *acc = sgg_mem + (size_t)g * CAP;
+    int *keys = (int *)(sgg_mem + (size_t)NG * CAP) + (size_t)g * 2 * CAP;
+    int *cols = (int *)(sgg_mem + (size_t)NG * CAP) + (size_t)NG * 2 * CAP + (size_t)g * CAP;
+    int *count = (int *)(sgg_mem + (size_t)NG * CAP) + (size_t)NG * 3 * CAP + g;
+    unsigned char *pos = (unsigned char *)((int *)(sgg_mem + (size_t)NG * CAP) + (size_t)NG * 3 * CAP + NG) +
+                         (size_t)g * 2 * CAP;
+    for (int t = lane; t < 2 * CAP / 4; t += G) reinterpret_cast<int4 *>(keys)[t] = make_int4(-1, -1, -1, -1);
+    // whole warps stay together (shuffles and barriers of the warp)
+    const long long step = (long long)gridDim.x * NG;
+    for (long long w0 = (long long)blockIdx.x * NG + (threadIdx.x / 32) * (32 / G); w0 < nr; w0 += step) {
+        const long long row = w0 + (threadIdx.x & 31) / G;
+        const bool live = row < nr && !(crp && crp[row + 1] - crp[row] > CAP);
+        const int e0 = live ? lrp[row] : 0, e1 = live ? lrp[row + 1] : 0;
+        if (lane == 0) *count = 0;
+        __syncwarp();
+        bool over = false;
+        for (int eb = e0; __any_sync(all, eb < e1 && !over); eb += G) {
+            int rs = 0, rl = 0;
+            double a = 0.0;
+            if (eb + lane < e1 && !over) {
+                const int k = lci[eb + lane];
+                a = lv[eb + lane];
+                rs = rrp[k];
+                rl = rrp[k + 1] - rs;
+            }
+            for (int t0 = 0; t0 < G && __any_sync(all, eb + t0 < e1 && !over); t0 += SGG_PF) {
+                int c[SGG_PF], n[SGG_PF], s[SGG_PF];
+                double v[SGG_PF];
+#pragma unroll
+                for (int t = 0; t < SGG_PF; ++t) {
+                    s[t] = __shfl_sync(all, rs, t0 + t, G);
+                    n[t] = __shfl_sync(all, rl, t0 + t, G);
+                    c[t] = 0;
+                    v[t] = 0.0;
+                    if (lane < n[t]) {
+                        c[t] = rci[s[t] + lane];
+                        v[t] = rv[s[t] + lane];
                     }
-                    list[pos * SGT_BS] = c;
-                    acc[pos * SGT_BS] = 0.0;
-                    ++u;
                 }
-                acc[pos * SGT_BS] = __dadd_rn(acc[pos * SGT_BS], __dmul_rn(a, rv[f]));
+                bool full = false;
+                // one product per lane: the lanes find their places, meet, and add
+                // (added where its search ended, a sum would take an FP64 instruction
+                // per distinct end of the search)
+                auto add = [&](bool on, int col, double prod) {
+                    const int p = on && !full ? sgg_find<CAP>(keys, pos, count, cols, acc, col) : CAP;
+                    __syncwarp();
+                    if (p < CAP) acc[p] = __dadd_rn(acc[p], prod);
+                    full = (__ballot_sync(all, full || (on && p >= CAP)) & mine) != 0;
+                };
+#pragma unroll
+                for (int t = 0; t < SGG_PF; ++t) {
+                    const double at = __shfl_sync(all, a, t0 + t, G);
+                    add(lane < n[t], c[t], __dmul_rn(at, v[t]));
+                    for (int f = lane + G; __any_sync(all, f < n[t]); f += G) {
+                        const bool on = f < n[t];
+                        add(on, on ? rci[s[t] + f] : 0, __dmul_rn(at, on ? rv[s[t] + f] : 0.0));
+                    }
+                }
+                over |= full;
             }
         }
-        for (int t = 0; t < u; ++t) {
-            cci[o + t] = list[t * SGT_BS];
-            cv[o + t] = acc[t * SGT_BS];
+        __syncwarp();
+        if (live) {
+            const int u = *count;
+            if (over) {
+                if (lane == 0) {
+                    long_rows[atomicAdd(nlong, 1)] = (int)row;
+                    cnt[row] = 0;
+                }
+            } else {
+                if (lane == 0 && !crp) cnt[row] = u;
+                const size_t base = crp ? (size_t)crp[row] : (size_t)row * CAP;
+                for (int p = lane; p < u && oci; p += G) {
+                    const int c = cols[p];
+                    int rank = 0;
+                    for (int q = 0; q < u; ++q) rank += cols[q] < c;
+                    oci[base + rank] = c;
+                    ov[base + rank] = acc[p];
+                }
+            }
+        }
+        __syncwarp();
+        for (int t = lane; t < 2 * CAP / 4; t += G) reinterpret_cast<int4 *>(keys)[t] = make_int4(-1, -1, -1, -1);
+    }
+}
+
+// the temporary's rows to their places; rows of more than cap entries are the
+// warp kernels'
+__global__ void k_sgg_pack(int nr, int cap, const int *__restrict__ crp, const int *__restrict__ tci,
+                           const double *__restrict__ tcv, int *__restrict__ cci, double *__restrict__ cv)
+{
+    const int lane = threadIdx.x & 7;
+    for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 8; r < nr;
+         r += (long long)gridDim.x * blockDim.x / 8) {
+        const int o = crp[r], u = crp[r + 1] - o;
+        if (u > cap) continue;
+        for (int k = lane; k < u; k += 8) {
+            cci[o + k] = tci[(size_t)r * cap + k];
+            cv[o + k] = tcv[(size_t)r * cap + k];
         }
     }
 }
 
 void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
 {
-    // 0: long rows, 1: their count, 2: largest distinct count of the short rows,
-    // 3: bound of the long rows, 4: overflow, 5: largest distinct count of the long rows
-    DBuf<int> ctr(6), long_rows;
+    // 0: count of the long rows, 1: bound of their products, 2: overflow,
+    // 3: their largest distinct count
+    DBuf<int> ctr(4), long_rows, tci;
+    DBuf<double> tcv;
     GW_CUDA(cudaMemsetAsync(ctr.p, 0, ctr.bytes(), st));
     C.nr = L.nr;
     C.nc = Rm.nc;
     C.rp.alloc((size_t)C.nr + 1);
-    // A thread a row pays off for many short rows (the level-0 products A P
-    // with about 24 products a row, 2M rows); with few rows or hundreds of
-    // products a row a warp a row is faster.  Products a row estimated from
-    // the mean row lengths.
-    const double per_row = L.nr ? (double)L.nnz / L.nr * ((double)Rm.nnz / std::max(1, Rm.nr)) : 0.0;
-    const bool thread_rows = setup_forms() ? setup_forms() == 1 : L.nr >= 32768 && per_row <= 128.0;
-    const int gt = nblk(L.nr, SGT_BS, 152LL * 64);
-    int nlong = L.nr, mu_short = 0;
-    if (thread_rows) {
-        long_rows.alloc((size_t)L.nr);
-        gw_launch(k_sgt_symbolic, gt, SGT_BS, 0, st, L.nr, L.rp.p, L.ci.p, Rm.rp.p, Rm.ci.p, C.rp.p, long_rows.p,
-                  ctr.p + 1, ctr.p + 2);
+    // Table and group by the mean products a row (of which 10-30 fall on one
+    // column on the fine levels) and the mean row length of Rm.  The warp form
+    // keeps products whose rows would mostly pass 128 columns.  Up to 4 GB of
+    // temporary (22 million fine cells) one run and a packing pass, 20 % of the
+    // run; beyond, two runs.
+    const double m = (double)Rm.nnz / std::max(1, Rm.nr), per_row = L.nr ? (double)L.nnz / L.nr * m : 0.0;
+    const int cap = per_row <= 40.0 ? 16 : per_row <= 1000.0 ? 64 : 128;
+    const bool groups = setup_forms() ? setup_forms() == 1 : per_row <= 16384.0;
+    const bool temp = (double)L.nr * cap * 12.0 <= SGG_TEMP_MAX;
+    auto run_groups = [&](const int *crp, int *cnt, int *oci, double *ov) {
+        auto run = [&](auto kernel, int G, size_t smem) {
+            // always the same value per kernel (see below)
+            GW_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            gw_launch(kernel, nblk((long long)L.nr * G, SGG_BS, 152LL * 64), SGG_BS, smem, st, L.nr, L.rp.p, L.ci.p,
+                      L.v.p, Rm.rp.p, Rm.ci.p, Rm.v.p, crp, cnt, oci, ov, long_rows.p, ctr.p);
+        };
+        if (cap == 16) run(k_sgg<4, 16>, 4, sgg_smem<4, 16>());
+        else if (cap == 128 && m <= 20.0) run(k_sgg<16, 128>, 16, sgg_smem<16, 128>());
+        else if (cap == 128) run(k_sgg<32, 128>, 32, sgg_smem<32, 128>());
+        else if (m <= 6.0) run(k_sgg<4, 64>, 4, sgg_smem<4, 64>());
+        else if (m <= 12.0) run(k_sgg<8, 64>, 8, sgg_smem<8, 64>());
+        else run(k_sgg<16, 64>, 16, sgg_smem<16, 64>());
         GW_LAUNCH_CHECK();
-        int hc[2];
-        GW_CUDA(cudaMemcpyAsync(hc, ctr.p + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
-        GW_CUDA(cudaStreamSynchronize(st));
-        nlong = hc[0];
-        mu_short = hc[1];
+    };
+    int nlong = L.nr;
+    if (groups) {
+        long_rows.alloc((size_t)L.nr);
+        if (temp) {
+            tci.alloc((size_t)L.nr * cap);
+            tcv.alloc((size_t)L.nr * cap);
+        }
+        run_groups(nullptr, C.rp.p, tci.p, tcv.p);
+        nlong = read_int(ctr.p, st);
     }
-    const int *rows = thread_rows ? (const int *)long_rows.p : nullptr;
+    const int *rows = groups ? (const int *)long_rows.p : nullptr;
     // The attribute is global to the kernel, and setups may run concurrently on
     // several threads: always set the same value, the largest any launch uses.
     GW_CUDA(cudaFuncSetAttribute(k_sg_symbolic, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM_MAX));
     GW_CUDA(cudaFuncSetAttribute(k_sg_numeric, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM_MAX));
     int Hn = 0, Wn = 0;
     if (nlong > 0) {
-        // rows with more than SGT_CAP distinct columns: a warp each
-        gw_launch(k_sg_bound, nblk(L.nr, 256), 256, 0, st, L.nr, Rm.nc, L.rp.p, L.ci.p, Rm.rp.p, ctr.p + 3);
+        // a warp each
+        gw_launch(k_sg_bound, nblk(L.nr, 256), 256, 0, st, L.nr, Rm.nc, L.rp.p, L.ci.p, Rm.rp.p, ctr.p + 1);
         GW_LAUNCH_CHECK();
-        const int ub = read_int(ctr.p + 3, st);
+        const int ub = read_int(ctr.p + 1, st);
         int H = 32;
         while (H < 2 * ub && H < SG_HMAX) H <<= 1;
         // warps per block so that a block's tables stay within 96 KB
@@ -1198,10 +1292,10 @@ void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
             fail(GW_ERR_SETUP, "SpGEMM shared memory %zu exceeds %d", smem_sym, SG_SMEM_MAX);
         const int grid = (int)std::max(1LL, std::min<long long>(((long long)nlong + W - 1) / W, 152LL * 64));
         gw_launch(k_sg_symbolic, grid, 32 * W, smem_sym, st, nlong, rows, L.rp.p, L.ci.p,
-                  Rm.rp.p, Rm.ci.p, H, C.rp.p, ctr.p + 4, ctr.p + 5);
+                  Rm.rp.p, Rm.ci.p, H, C.rp.p, ctr.p + 2, ctr.p + 3);
         GW_LAUNCH_CHECK();
         int hl[2];
-        GW_CUDA(cudaMemcpyAsync(hl, ctr.p + 4, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+        GW_CUDA(cudaMemcpyAsync(hl, ctr.p + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
         GW_CUDA(cudaStreamSynchronize(st));
         if (hl[0]) fail(GW_ERR_SETUP, "SpGEMM row has more than %d distinct columns", H / 2);
         // the numeric pass knows every row's distinct count: tables of twice the largest
@@ -1216,15 +1310,11 @@ void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
     C.nnz = read_int(C.rp.p + C.nr, st);
     C.ci.alloc((size_t)C.nnz);
     C.v.alloc((size_t)C.nnz);
-    if (mu_short > 0) {
-        auto numeric = [&](auto kernel, int cap) {
-            GW_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SGT_CAP * SGT_BS * 12));
-            gw_launch(kernel, gt, SGT_BS, (size_t)cap * SGT_BS * 12, st, L.nr, L.rp.p, L.ci.p, L.v.p, Rm.rp.p,
-                      Rm.ci.p, Rm.v.p, C.rp.p, C.ci.p, C.v.p);
-        };
-        if (mu_short <= 16) numeric(k_sgt_numeric<16>, 16);
-        else if (mu_short <= 32) numeric(k_sgt_numeric<32>, 32);
-        else numeric(k_sgt_numeric<SGT_CAP>, SGT_CAP);
+    if (groups && !temp) {
+        run_groups(C.rp.p, nullptr, C.ci.p, C.v.p);
+    } else if (groups && nlong < L.nr) {
+        gw_launch(k_sgg_pack, nblk((long long)L.nr * 8, 256, 152LL * 64), 256, 0, st, L.nr, cap, C.rp.p, tci.p, tcv.p,
+                  C.ci.p, C.v.p);
         GW_LAUNCH_CHECK();
     }
     if (nlong > 0) {
