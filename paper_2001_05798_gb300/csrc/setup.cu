@@ -1508,8 +1508,11 @@ void setup_dense_inverse(const DCSR &A, DBuf<double> &Ainv, cudaStream_t st)
 }
 
 // ------------------------------------------------- smoother data (per level) --
+// diagonal, its inverse (for the power iteration and the smoother's weights),
+// and the largest Gershgorin ratio
 __global__ void k_gersh(int n, const int *__restrict__ rp, const int *__restrict__ ci, const double *__restrict__ v,
-                        double *__restrict__ d, unsigned long long *__restrict__ rho_bits)
+                        double *__restrict__ d, double *__restrict__ inv,
+                        unsigned long long *__restrict__ rho_bits)
 {
     unsigned long long best = 0;
     GRID_STRIDE(ii, n)
@@ -1521,6 +1524,7 @@ __global__ void k_gersh(int n, const int *__restrict__ rp, const int *__restrict
             if (ci[e] == i) dd = v[e];
         }
         d[i] = dd;
+        inv[i] = 1.0 / dd;
         const double ratio = s / dd;
         if (ratio > 0.0 && isfinite(ratio)) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(ratio);
@@ -1530,12 +1534,13 @@ __global__ void k_gersh(int n, const int *__restrict__ rp, const int *__restrict
     block_atomic_max(best, rho_bits);
 }
 
-double setup_gershgorin(const DCSR &A, DBuf<double> &diag, cudaStream_t st)
+double setup_gershgorin(const DCSR &A, DBuf<double> &diag, DBuf<double> &inv, cudaStream_t st)
 {
     diag.alloc((size_t)A.nr);
+    inv.alloc((size_t)A.nr);
     DBuf<unsigned long long> rb(1);
     GW_CUDA(cudaMemsetAsync(rb.p, 0, sizeof(unsigned long long), st));
-    gw_launch(k_gersh, nblk(A.nr, 256), 256, 0, st, A.nr, A.rp.p, A.ci.p, A.v.p, diag.p, rb.p);
+    gw_launch(k_gersh, nblk(A.nr, 256), 256, 0, st, A.nr, A.rp.p, A.ci.p, A.v.p, diag.p, inv.p, rb.p);
     GW_LAUNCH_CHECK();
     unsigned long long bits = 0;
     GW_CUDA(cudaMemcpyAsync(&bits, rb.p, sizeof bits, cudaMemcpyDeviceToHost, st));
@@ -1555,10 +1560,13 @@ __global__ void k_pow_start(int n, uint64_t seed, int level, double *__restrict_
     }
 }
 
-// w = D^-1 A v and per-block partial sums of w.w; G lanes a row
+// w = D^-1 A v and per-block partial sums of w.w; G lanes a row.  The inverse of
+// the diagonal comes in: an FP64 division is some dozen FP64 instructions, 16
+// issue cycles each on this GPU, against 7 multiply-adds of a level-0 row (160^3:
+// 138 us a step with the division on level 0, 113 on level 1).
 template <int G>
 __global__ void __launch_bounds__(256) k_pow_step(int n, const int *__restrict__ rp, const int *__restrict__ ci,
-                                                  const double *__restrict__ a, const double *__restrict__ d,
+                                                  const double *__restrict__ a, const double *__restrict__ inv,
                                                   const double *__restrict__ v, double *__restrict__ w,
                                                   double *__restrict__ part)
 {
@@ -1576,7 +1584,7 @@ __global__ void __launch_bounds__(256) k_pow_step(int n, const int *__restrict__
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off, G);
         if (lane == 0 && ii < n) {
-            s /= d[i];
+            s *= inv[i];
             w[i] = s;
             loc += s * s;
         }
@@ -1595,7 +1603,7 @@ __global__ void __launch_bounds__(256) k_pow_step(int n, const int *__restrict__
 // a few units at most, so ten steps stay far from overflow), and
 // lambda = |x_10| / |x_9|, the same estimate as normalised iterations give.
 // The ten steps run back to back; the host reads the two last norms once.
-double setup_power_lambda(const DCSR &A, const double *diag, uint64_t seed, int level, cudaStream_t st)
+double setup_power_lambda(const DCSR &A, const double *inv, uint64_t seed, int level, cudaStream_t st)
 {
     const int n = A.nr;
     const double per_row = n ? (double)A.nnz / n : 0.0;
@@ -1606,9 +1614,9 @@ double setup_power_lambda(const DCSR &A, const double *diag, uint64_t seed, int 
     GW_LAUNCH_CHECK();
     for (int it = 0; it < 10; ++it) {
         double *pp = part.p + (size_t)(it & 1) * g;
-        if (G == 1) gw_launch(k_pow_step<1>, g, 256, 0, st, n, A.rp.p, A.ci.p, A.v.p, diag, v.p, w.p, pp);
-        else if (G == 8) gw_launch(k_pow_step<8>, g, 256, 0, st, n, A.rp.p, A.ci.p, A.v.p, diag, v.p, w.p, pp);
-        else gw_launch(k_pow_step<32>, g, 256, 0, st, n, A.rp.p, A.ci.p, A.v.p, diag, v.p, w.p, pp);
+        if (G == 1) gw_launch(k_pow_step<1>, g, 256, 0, st, n, A.rp.p, A.ci.p, A.v.p, inv, v.p, w.p, pp);
+        else if (G == 8) gw_launch(k_pow_step<8>, g, 256, 0, st, n, A.rp.p, A.ci.p, A.v.p, inv, v.p, w.p, pp);
+        else gw_launch(k_pow_step<32>, g, 256, 0, st, n, A.rp.p, A.ci.p, A.v.p, inv, v.p, w.p, pp);
         GW_LAUNCH_CHECK();
         std::swap(v, w);
     }
