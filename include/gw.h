@@ -224,9 +224,8 @@ int gw_matrix_export(gw_matrix A, int *rowptr, int *col, double *val, void *stre
  * gw_amg_setup -- the AMG setup phase (Introduction): strength graph,
  * deterministic parallel MIS-2 aggregation with hashed seeded priorities,
  * tentative prolongator, one damped-Jacobi smoothing of it, Galerkin coarse
- * operators A_{l+1} = P^T A_l P by a two-pass SpGEMM, and a dense inverse of
- * the (SPD) coarsest level by block Gauss-Jordan elimination without
- * pivoting; then the V-cycle storage in the chosen precision.  All of it
+ * operators A_{l+1} = P^T A_l P by SpGEMM, and a dense inverse of the (SPD)
+ * coarsest level by a block sweep without pivoting; then the V-cycle storage in the chosen precision.  All of it
  * runs in CUDA kernels.  The aggregates and the P and A_{l+1} patterns and
  * values are the same as a serial FP64 implementation that sums in the
  * stated order (no fused multiply-add in these stages).

@@ -1328,24 +1328,29 @@ void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
 }
 
 // ---------------------------------------------------------- coarsest level --
-// Dense inverse of the coarsest level by block Gauss-Jordan elimination in
-// place, without pivoting (the coarsest operator is a Galerkin product of
-// the SPD level-0 operator with a full-rank prolongator, so it is SPD, and
-// elimination without pivoting is stable on SPD matrices; a pivot that is
-// not positive and finite reports the matrix as singular).  M (n x n,
-// row-major) starts as A; for each panel K of GJB consecutive indices:
-//   Q = (M_KK)^-1,
-//   M_IJ -= M_IK Q M_KJ  (I, J outside K),
-//   M_KJ  = Q M_KJ,  M_IK = -M_IK Q,  M_KK = Q,
-// and after the last panel M = A^-1.  Each panel is two launches: one block
-// per 32-column tile J inverts M_KK (every block the same way, in shared
-// memory), forms the new row panel Q M_KJ and copies the old column panel
-// M_JK aside; then one block per 32 x 32 tile of M applies the update.  The
-// n^3 FP64 multiply-adds so run on every SM, in 2 n / GJB launches.  The
-// launches run back to back with programmatic dependent launch: each kernel
+// Dense inverse of the coarsest level by the block sweep operator, in place and
+// without pivoting (the coarsest operator is a Galerkin product of the SPD
+// level-0 operator with a full-rank prolongator, so it is SPD, and elimination
+// without pivoting is stable on SPD matrices; a pivot that is not positive and
+// finite reports the matrix as singular).  M (n x n, row-major) starts as A; for
+// each panel K of GJB consecutive indices, with Q = (M_KK)^-1 and T_I = M_IK Q:
+//   M_IJ -= T_I M_KJ  (I, J outside K),  M_IK = T_I,  M_KJ = T_J^T,  M_KK = -Q,
+// which keeps M symmetric and leaves -A^-1 (Goodnight 1979); the last panel
+// writes the negative.  Symmetry halves the n^3 FP64 multiply-adds: a tile
+// (I, J), I >= J, is computed once and written in both places.
+// Two launches a panel: T and a copy of the old column panel (a block per
+// 16 rows), then the tiles.  The block of the next panel's diagonal tile comes
+// first and inverts it when it has it, while the other tiles run, so that the
+// 16 dependent steps of an inverse (some 0.4 us each: an FP64 division, then 8
+// warps' multiply-adds at 16 cycles each) are the only ones that nothing hides.
+// 16 indices a panel: a 32-index tile product holds an SM's FP64 units for 8.6 us,
+// and a coarsest level of a few hundred unknowns has too few of them for 152 SMs
+// (against block Gauss-Jordan on the whole matrix with 32-index panels a 45^3
+// request, some 310 unknowns, went from 5.61 to 5.38 ms, 160^3 from 31.3 to 30.9).
+// The launches run back to back with programmatic dependent launch: each kernel
 // may be scheduled while its predecessor runs and waits for it (and its
 // writes) before touching memory.
-constexpr int GJB = 32;
+constexpr int GJB = 16;
 
 __device__ __forceinline__ void gj_enter()
 {
@@ -1369,109 +1374,115 @@ static void gj_launch(void (*kernel)(KArgs...), int grid, int block, cudaStream_
     GW_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
 }
 
-// Inverse of the bk x bk pivot block in shared memory (row stride GJB+1),
-// in-place Gauss-Jordan without pivoting; 256 threads.  Returns false (for
-// every thread) if a pivot is not positive and finite.
-__device__ bool gj_invert_block(double (*a)[GJB + 1], double *col, int bk)
+// Inverse of a bk x bk pivot block held one entry a thread (thread (i, j) of the
+// 16 x 16 block has a, identity beyond bk), by Gauss-Jordan without pivoting.
+// Returns false (for every thread) if a pivot is not positive and finite.
+__device__ bool gj_invert_block(double &a, int i, int j, int bk)
 {
-    const int tid = threadIdx.x;
-    __shared__ int bad;
-    if (tid == 0) bad = 0;
-    __syncthreads();
+    __shared__ double row[2][GJB], col[2][GJB], rp[2];
     for (int p = 0; p < bk; ++p) {
-        const double piv = a[p][p];
-        if (!(piv > 0.0) || !isfinite(piv)) {
-            if (tid == 0) bad = 1;
-            break;  // uniform: every thread read the same pivot
-        }
-        if (tid < bk) col[tid] = a[tid][p];
+        const int s = p & 1;  // two sets of buffers: one barrier a step
+        if (i == p) row[s][j] = a;
+        if (j == p) col[s][i] = a;
+        if (i == p && j == p) rp[s] = 1.0 / a;
         __syncthreads();
-        // row p scaled by 1/piv, with its diagonal entry replaced by 1/piv
-        if (tid < bk) a[p][tid] = (tid == p ? 1.0 : a[p][tid]) / piv;
-        __syncthreads();
-        for (int t = tid; t < bk * bk; t += blockDim.x) {
-            const int i = t / bk, j = t % bk;
-            if (i != p) a[i][j] = (j == p ? 0.0 : a[i][j]) - col[i] * a[p][j];
-        }
-        __syncthreads();
+        const double piv = row[s][p], r = rp[s];
+        if (!(piv > 0.0) || !isfinite(piv)) return false;  // uniform: every thread read the same pivot
+        const double t = (i == p ? 1.0 : row[s][j]) * r;
+        if (i == p) a = j == p ? r : row[s][j] * r;
+        else a = j == p ? -(col[s][i] * r) : fma(-col[s][i], t, a);
     }
-    __syncthreads();
-    return bad == 0;
+    return true;
 }
 
-// One block per 32-index tile J: Q = (M_KK)^-1, Rn[:, J] = Q M_KJ, Cs[J, :]
-// = M_JK (old values); block 0 also stores Q.
-__global__ void __launch_bounds__(256) k_bgj_panel(int n, int k0, int bk, const double *__restrict__ M,
-                                                   double *__restrict__ Q, double *__restrict__ Rn,
-                                                   double *__restrict__ Cs, int *__restrict__ singular)
+// Q of the first panel (one block)
+__global__ void __launch_bounds__(256) k_sweep_pivot(int n, int bk, const double *__restrict__ M,
+                                                     double *__restrict__ Q, int *__restrict__ singular)
 {
-    __shared__ double a[GJB][GJB + 1], t[GJB][GJB + 1];
-    __shared__ double col[GJB];
-    const int tid = threadIdx.x, j0 = blockIdx.x * GJB, bj = min(GJB, n - j0);
+    const int i = threadIdx.x / GJB, j = threadIdx.x % GJB;
     gj_enter();
-    if (*(volatile const int *)singular) return;
-    for (int e = tid; e < GJB * GJB; e += blockDim.x) {
-        const int i = e / GJB, j = e % GJB;
-        a[i][j] = i < bk && j < bk ? M[(size_t)(k0 + i) * n + k0 + j] : 0.0;
-        t[i][j] = i < bk && j < bj ? M[(size_t)(k0 + i) * n + j0 + j] : 0.0;
-    }
-    __syncthreads();
-    // old column panel rows of this tile
-    for (int e = tid; e < GJB * GJB; e += blockDim.x) {
-        const int i = e / GJB, j = e % GJB;
-        if (i < bj && j < bk) Cs[(size_t)(j0 + i) * GJB + j] = M[(size_t)(j0 + i) * n + k0 + j];
-    }
-    if (!gj_invert_block(a, col, bk)) {
-        if (tid == 0) atomicExch(singular, 1);
+    double a = i < bk && j < bk ? M[(size_t)i * n + j] : (i == j ? 1.0 : 0.0);
+    if (!gj_invert_block(a, i, j, bk)) {
+        if (threadIdx.x == 0) atomicExch(singular, 1);
         return;
     }
-    if (blockIdx.x == 0)
-        for (int e = tid; e < GJB * GJB; e += blockDim.x) Q[e] = a[e / GJB][e % GJB];
-    // Rn[:, J] = Q M_KJ, terms in ascending inner index
-    for (int e = tid; e < bk * bj; e += blockDim.x) {
-        const int i = e / bj, j = e % bj;
-        double s = 0.0;
-        for (int q = 0; q < bk; ++q) s = fma(a[i][q], t[q][j], s);
-        Rn[(size_t)i * n + j0 + j] = s;
-    }
+    Q[threadIdx.x] = i < bk && j < bk ? a : 0.0;
 }
 
-// One block per 32 x 32 tile (I, J) of M: the panel update above.
-__global__ void __launch_bounds__(256) k_bgj_update(int n, int k0, int bk, double *__restrict__ M,
-                                                    const double *__restrict__ Q, const double *__restrict__ Rn,
-                                                    const double *__restrict__ Cs, const int *__restrict__ singular)
+// One block per 16 rows I: Cs[I, :] = M_IK (old values), T[I, :] = M_IK Q
+__global__ void __launch_bounds__(256) k_sweep_panel(int n, int k0, int bk, const double *__restrict__ M,
+                                                     const double *__restrict__ Q, double *__restrict__ T,
+                                                     double *__restrict__ Cs, const int *__restrict__ singular)
 {
-    __shared__ double c[GJB][GJB + 1], r[GJB][GJB + 1];
-    const int tid = threadIdx.x;
-    const int nt = (n + GJB - 1) / GJB;
-    const int ti = blockIdx.x / nt, tj = blockIdx.x % nt;
-    const int i0 = ti * GJB, j0 = tj * GJB, bi = min(GJB, n - i0), bj = min(GJB, n - j0);
-    const int kt = k0 / GJB;
+    __shared__ double c[GJB][GJB + 1], q[GJB][GJB + 1];
+    const int i = threadIdx.x / GJB, j = threadIdx.x % GJB, row = blockIdx.x * GJB + i;
     gj_enter();
     if (*(volatile const int *)singular) return;
-    if (ti == kt && tj == kt) {
-        for (int e = tid; e < bk * bk; e += blockDim.x)
-            M[(size_t)(k0 + e / bk) * n + k0 + e % bk] = Q[(e / bk) * GJB + e % bk];
-        return;
-    }
-    if (ti == kt) {
-        for (int e = tid; e < bk * bj; e += blockDim.x)
-            M[(size_t)(k0 + e / bj) * n + j0 + e % bj] = Rn[(size_t)(e / bj) * n + j0 + e % bj];
-        return;
-    }
-    // c = old M_IK (bi x bk); r = Rn[:, J] (bk x bj), or Q for the tile in column K
-    for (int e = tid; e < GJB * GJB; e += blockDim.x) {
-        const int i = e / GJB, j = e % GJB;
-        c[i][j] = i < bi && j < bk ? Cs[(size_t)(i0 + i) * GJB + j] : 0.0;
-        r[i][j] = i < bk && j < bj ? (tj == kt ? Q[i * GJB + j] : Rn[(size_t)i * n + j0 + j]) : 0.0;
-    }
+    const double m = row < n && j < bk ? M[(size_t)row * n + k0 + j] : 0.0;
+    c[i][j] = m;
+    q[i][j] = Q[threadIdx.x];
     __syncthreads();
-    for (int e = tid; e < bi * bj; e += blockDim.x) {
-        const int i = e / bj, j = e % bj;
-        double s = 0.0;
-        for (int q = 0; q < bk; ++q) s = fma(c[i][q], r[q][j], s);
-        double *m = M + (size_t)(i0 + i) * n + j0 + j;
-        *m = tj == kt ? -s : *m - s;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < GJB; ++k) s = fma(c[i][k], q[k][j], s);
+    Cs[(size_t)blockIdx.x * GJB * GJB + threadIdx.x] = m;
+    T[(size_t)blockIdx.x * GJB * GJB + threadIdx.x] = s;
+}
+
+// One block per tile (I, J), I >= J: the panel update above; Qn: Q of the next
+// panel.  neg: the last panel, whose results are written negated.
+__global__ void __launch_bounds__(256) k_sweep_update(int n, int k0, int bk, double *__restrict__ M,
+                                                      const double *__restrict__ Q, const double *__restrict__ T,
+                                                      const double *__restrict__ Cs, double *__restrict__ Qn, int neg,
+                                                      int *__restrict__ singular)
+{
+    __shared__ double t[GJB][GJB + 1], c[GJB][GJB + 1];
+    const int i = threadIdx.x / GJB, j = threadIdx.x % GJB, K = k0 / GJB;
+    const int next = (K + 1) * (K + 2) / 2 + K + 1;  // tile (K + 1, K + 1), first
+    int b = blockIdx.x;
+    if (next < (int)gridDim.x) b = b == 0 ? next : b == next ? 0 : b;
+    int I = (int)((sqrtf(8.0f * b + 1.0f) - 1.0f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= b) ++I;
+    while (I * (I + 1) / 2 > b) --I;
+    const int J = b - I * (I + 1) / 2;
+    const double sg = neg ? -1.0 : 1.0;
+    gj_enter();
+    if (*(volatile const int *)singular) return;
+    const int r = I * GJB + i, s = J * GJB + j;
+    double v;
+    if (I == K && J == K) {
+        v = -Q[threadIdx.x];
+    } else if (I == K) {
+        v = T[(size_t)J * GJB * GJB + j * GJB + i];  // M_KJ = T_J^T
+    } else if (J == K) {
+        v = T[(size_t)I * GJB * GJB + threadIdx.x];
+    } else {
+        v = r < n && s < n ? M[(size_t)r * n + s] : 0.0;
+        t[i][j] = T[(size_t)I * GJB * GJB + threadIdx.x];
+        c[i][j] = Cs[(size_t)J * GJB * GJB + threadIdx.x];
+        __syncthreads();
+        double x = 0.0;
+#pragma unroll
+        for (int k = 0; k < GJB; ++k) x = fma(t[i][k], c[j][k], x);
+        v -= x;
+        __syncthreads();
+    }
+    // the transposed tile through shared memory; on the diagonal the lower half
+    // stands for both
+    t[i][j] = v;
+    __syncthreads();
+    if (I == J) v = i >= j ? v : t[j][i];
+    if (r < n && s < n) M[(size_t)r * n + s] = sg * v;
+    const int r2 = J * GJB + i, s2 = I * GJB + j;
+    if (I != J && r2 < n && s2 < n) M[(size_t)r2 * n + s2] = sg * t[j][i];
+    if (I == K + 1 && J == K + 1) {
+        const int bn = min(GJB, n - (K + 1) * GJB);
+        double a = i < bn && j < bn ? v : (i == j ? 1.0 : 0.0);
+        if (!gj_invert_block(a, i, j, bn)) {
+            if (threadIdx.x == 0) atomicExch(singular, 1);
+            return;
+        }
+        Qn[threadIdx.x] = i < bn && j < bn ? a : 0.0;
     }
 }
 
@@ -1490,18 +1501,21 @@ void setup_dense_inverse(const DCSR &A, DBuf<double> &Ainv, cudaStream_t st)
     const int n = A.nr;
     if (n > 4096) fail(GW_ERR_SETUP, "coarsest level has %d unknowns (more than 4096)", n);
     const int nt = (n + GJB - 1) / GJB;
-    DBuf<double> Q((size_t)GJB * GJB), Rn((size_t)GJB * n), Cs((size_t)nt * GJB * GJB);
+    constexpr size_t TILE = (size_t)GJB * GJB;
+    DBuf<double> Q(2 * TILE), T((size_t)nt * TILE), Cs((size_t)nt * TILE);
     DBuf<int> sing(1);
     Ainv.alloc((size_t)n * n);
     GW_CUDA(cudaMemsetAsync(Ainv.p, 0, Ainv.bytes(), st));
     GW_CUDA(cudaMemsetAsync(sing.p, 0, sizeof(int), st));
     gw_launch(k_gj_fill, nblk(n, 128), 128, 0, st, n, A.rp.p, A.ci.p, A.v.p, Ainv.p);
     GW_LAUNCH_CHECK();
-    for (int k0 = 0; k0 < n; k0 += GJB) {
-        const int bk = std::min(GJB, n - k0);
-        gj_launch(k_bgj_panel, nt, 256, st, n, k0, bk, (const double *)Ainv.p, Q.p, Rn.p, Cs.p, (int *)sing.p);
-        gj_launch(k_bgj_update, nt * nt, 256, st, n, k0, bk, Ainv.p, (const double *)Q.p, (const double *)Rn.p,
-                  (const double *)Cs.p, (const int *)sing.p);
+    gj_launch(k_sweep_pivot, 1, 256, st, n, std::min(GJB, n), (const double *)Ainv.p, Q.p, (int *)sing.p);
+    for (int K = 0; K < nt; ++K) {
+        const int k0 = K * GJB, bk = std::min(GJB, n - k0);
+        const double *q = Q.p + (size_t)(K & 1) * TILE;
+        gj_launch(k_sweep_panel, nt, 256, st, n, k0, bk, (const double *)Ainv.p, q, T.p, Cs.p, (const int *)sing.p);
+        gj_launch(k_sweep_update, nt * (nt + 1) / 2, 256, st, n, k0, bk, Ainv.p, q, (const double *)T.p,
+                  (const double *)Cs.p, Q.p + (size_t)((K + 1) & 1) * TILE, K + 1 == nt ? 1 : 0, (int *)sing.p);
     }
     GW_LAUNCH_CHECK();
     if (read_int(sing.p, st)) fail(GW_ERR_SETUP, "coarsest-level matrix (%d unknowns) is singular", n);
