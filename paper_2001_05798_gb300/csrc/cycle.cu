@@ -2456,8 +2456,12 @@ __device__ __forceinline__ void with_bmat(const BMat &m, F f)
     }
 }
 
+// Four resident blocks a SM (64 registers): with every matrix form's body in one
+// kernel the compiler took 128-174 registers, one or two blocks, which cannot hide
+// the latencies of an item's start.  Eight solves of sides 33-96: 16.2 -> 14.1 ms
+// (with five blocks 16.4: spills).
 template <int KIND>
-__global__ void __launch_bounds__(BS) kb_pass(const BSlot *__restrict__ slots, const int4 *__restrict__ work,
+__global__ void __launch_bounds__(BS, 4) kb_pass(const BSlot *__restrict__ slots, const int4 *__restrict__ work,
                                               const int *__restrict__ wcnt, int launch, BLaunch Lc)
 {
     pdl_enter();
