@@ -584,6 +584,53 @@ struct MStenH {
     }
 };
 
+// Least resident blocks a SM asked of the compiler for a pass (the second launch
+// bound; 0: none).  These passes are bound by the latency of their loads, and
+// without the bound ptxas keeps the registers low (32-62, 4-8 blocks) by issuing a
+// thread's loads late; asked for few blocks it keeps the loads of both unrolled
+// row groups, or of all neighbours, in flight, which hides more than the blocks
+// lost.  Measured per pass (us, without -> with): FP32 stencil of 4 rows a thread
+// at 128^3, CG product 17.2 -> 15.1, last post-smoothing step 17.3 -> 16.0, residual
+// 8.7 -> 6.7, first post-smoothing step 11.5 -> 11.0 (three blocks), pre-smoothing
+// 10.8 -> 12.7 (so none there).  One or two rows a thread: 117^3 solve 7.26 -> 6.75 ms;
+// FP64 at 96^3: stencil 10.2 -> 9.2, sliced ELL 9.2 -> 8.8 ms; BF16 and FP16
+// stencils 27.1 -> 26.9 ms at 256x256x128.  The FP32 sliced ELL lost (level 1 of
+// 128^3 is 737 blocks: five a SM are one wave, four are two).
+enum { PASS_ZERO2, PASS_CHEB0, PASS_OTHER };
+template <class M>
+struct MinBlocks {
+    static constexpr int at(int) { return 0; }
+};
+template <>
+struct MinBlocks<MSten<float, 4>> {
+    static constexpr int at(int pass) { return pass == PASS_ZERO2 ? 0 : pass == PASS_CHEB0 ? 3 : 2; }
+};
+template <>
+struct MinBlocks<MSten<float, 2>> {
+    static constexpr int at(int) { return 1; }
+};
+template <>
+struct MinBlocks<MSten<float, 1>> {
+    static constexpr int at(int) { return 1; }
+};
+template <int R>
+struct MinBlocks<MStenB<R>> {
+    static constexpr int at(int) { return 1; }
+};
+template <int R>
+struct MinBlocks<MStenH<R>> {
+    static constexpr int at(int) { return 1; }
+};
+template <int R>
+struct MinBlocks<MSten<double, R>> {
+    static constexpr int at(int) { return 3; }
+};
+template <int G>
+struct MinBlocks<MSell<double, G>> {
+    static constexpr int at(int) { return 2; }
+};
+#define PASS_BOUNDS(M, pass) __launch_bounds__(BS, MinBlocks<M>::at(pass))
+
 // rows per thread of the level-0 stencil: 4 (16 bytes of FP32, 32 bytes of
 // FP64 per array); 8 FP32 rows per thread measured slower (more registers,
 // fewer resident blocks)
@@ -747,7 +794,7 @@ __device__ __forceinline__ void b_jac0_res(VB vb, M A, int n, const typename M::
 }
 
 template <class M, class BT>
-__global__ void __launch_bounds__(BS) k_jac0_res(M A, int n, const typename M::value_type *__restrict__ dw,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_jac0_res(M A, int n, const typename M::value_type *__restrict__ dw,
                                                  const BT *__restrict__ b, typename M::value_type *__restrict__ x,
                                                  typename M::value_type *__restrict__ r, const Ctl *ctl)
 {
@@ -791,7 +838,7 @@ __device__ __forceinline__ void b_jacobi(VB vb, M A, int n, const typename M::va
 }
 
 template <class M, class BT, class OT, bool DOT>
-__global__ void __launch_bounds__(BS) k_jacobi(M A, int n, const typename M::value_type *__restrict__ dw,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_jacobi(M A, int n, const typename M::value_type *__restrict__ dw,
                                                const BT *__restrict__ b, const typename M::value_type *__restrict__ xi,
                                                OT *__restrict__ xo, const typename M::value_type *__restrict__ q,
                                                double *part, Ctl *ctl, int mode)
@@ -822,7 +869,7 @@ __device__ __forceinline__ void b_residual(VB vb, M A, int n, const BT *__restri
 }
 
 template <class M, class BT>
-__global__ void __launch_bounds__(BS) k_residual(M A, int n, const BT *__restrict__ b,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_residual(M A, int n, const BT *__restrict__ b,
                                                  const typename M::value_type *__restrict__ x,
                                                  typename M::value_type *__restrict__ r, const Ctl *ctl)
 {
@@ -870,7 +917,7 @@ __device__ __forceinline__ void b_spmv(VB vb, M Rm, int n, const typename M::val
 }
 
 template <class M>
-__global__ void __launch_bounds__(BS) k_spmv(M Rm, int n, const typename M::value_type *__restrict__ x,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_spmv(M Rm, int n, const typename M::value_type *__restrict__ x,
                                              typename M::value_type *__restrict__ y,
                                              First<typename M::value_type> f, const Ctl *ctl)
 {
@@ -898,7 +945,7 @@ __device__ __forceinline__ void b_prolong(VB vb, M P, int n, const typename M::v
 }
 
 template <class M>
-__global__ void __launch_bounds__(BS) k_prolong(M P, int n, const typename M::value_type *__restrict__ e,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_prolong(M P, int n, const typename M::value_type *__restrict__ e,
                                                 typename M::value_type *__restrict__ x, const Ctl *ctl)
 {
     pdl_enter();
@@ -1107,7 +1154,7 @@ __device__ __forceinline__ void b_restrict_sum(VB vb, int nc, const int *__restr
     }
 }
 
-__global__ void __launch_bounds__(BS) k_restrict_sum(int nc, const int *__restrict__ mptr, const int *__restrict__ mem,
+__global__ void __launch_bounds__(BS, 2) k_restrict_sum(int nc, const int *__restrict__ mptr, const int *__restrict__ mem,
                                                      const float *__restrict__ u, float *__restrict__ rc,
                                                      const Ctl *ctl)
 {
@@ -1209,7 +1256,7 @@ __device__ __forceinline__ void b_cheb0(VB vb, M A, int n, const typename M::val
 }
 
 template <class M, class BT, class OT, bool DOT>
-__global__ void __launch_bounds__(BS) k_cheb0(M A, int n, const typename M::value_type *__restrict__ dw,
+__global__ void PASS_BOUNDS(M, PASS_CHEB0) k_cheb0(M A, int n, const typename M::value_type *__restrict__ dw,
                                               const BT *__restrict__ b, typename M::value_type *x,
                                               typename M::value_type *__restrict__ r,
                                               typename M::value_type *__restrict__ d, OT *__restrict__ xo,
@@ -1277,7 +1324,7 @@ __device__ __forceinline__ void b_chebk(VB vb, M A, int n, const typename M::val
 }
 
 template <class M, class OT, bool DOT>
-__global__ void __launch_bounds__(BS) k_chebk(M A, int n, const typename M::value_type *__restrict__ dw,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_chebk(M A, int n, const typename M::value_type *__restrict__ dw,
                                               typename M::value_type *__restrict__ r,
                                               const typename M::value_type *__restrict__ d,
                                               typename M::value_type *__restrict__ dn, typename M::value_type *x,
@@ -1353,7 +1400,7 @@ __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M
 }
 
 template <class M, class OT, bool DOT, bool PRE>
-__global__ void __launch_bounds__(BS) k_cheb_zero2(M A, int n, const typename M::value_type *__restrict__ dw,
+__global__ void PASS_BOUNDS(M, PASS_ZERO2) k_cheb_zero2(M A, int n, const typename M::value_type *__restrict__ dw,
                                                    const typename M::value_type *__restrict__ b,
                                                    typename M::value_type *__restrict__ x,
                                                    typename M::value_type *__restrict__ r,
@@ -1739,7 +1786,7 @@ __global__ void __launch_bounds__(BS) k_copy(int n, const V *__restrict__ a, V *
 
 // q = A p, pq = (p, q); alpha = rz / pq
 template <class M>
-__global__ void __launch_bounds__(BS) k_cg_spmv_dot(M A, int n, const typename M::value_type *__restrict__ p,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_cg_spmv_dot(M A, int n, const typename M::value_type *__restrict__ p,
                                                     typename M::value_type *__restrict__ q, double *part, Ctl *c)
 {
     const VB vb = vb_grid();
@@ -1825,7 +1872,7 @@ __device__ __forceinline__ void b_cg_dir_spmv(VB vb, M A, int n, const typename 
 }
 
 template <class M>
-__global__ void __launch_bounds__(BS) k_cg_dir_spmv(M A, int n, const typename M::value_type *__restrict__ z,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_cg_dir_spmv(M A, int n, const typename M::value_type *__restrict__ z,
                                                     typename M::value_type *pa, typename M::value_type *pb,
                                                     typename M::value_type *__restrict__ q, double *part, Ctl *c)
 {
@@ -1847,7 +1894,8 @@ __device__ __forceinline__ void b_cg_update(VB vb, int n, V *__restrict__ x, V *
     DAcc acc[1];
     // two of the thread's row groups per step, all their loads issued first
     // (the second group's loads no longer wait for the first's); the groups
-    // are added to the dot in the same order as one at a time
+    // are added to the dot in the same order as one at a time.  The launch bound
+    // of two blocks lets the compiler hold them all (128^3: 12.8 -> 11.0 us)
     const int stride = R * vb.nb * BS;
     for (int i = R * (vb.bid * BS + threadIdx.x); i < n; i += 2 * stride) {
         const int i2 = i + stride;
@@ -1892,7 +1940,7 @@ __device__ __forceinline__ void b_cg_update(VB vb, int n, V *__restrict__ x, V *
 }
 
 template <class V, int R>
-__global__ void __launch_bounds__(BS) k_cg_update(int n, V *__restrict__ x, V *__restrict__ r, const V *pa,
+__global__ void __launch_bounds__(BS, 2) k_cg_update(int n, V *__restrict__ x, V *__restrict__ r, const V *pa,
                                                   const V *pb, const V *__restrict__ q, double *part, Ctl *c,
                                                   int reliable)
 {
@@ -1902,7 +1950,7 @@ __global__ void __launch_bounds__(BS) k_cg_update(int n, V *__restrict__ x, V *_
 
 // FP64 form: when the recursive residual passed, r = b - A x; stop if it passes too
 template <class M>
-__global__ void __launch_bounds__(BS) k_cg_true(M A, int n, const double *__restrict__ b, const double *__restrict__ x,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_cg_true(M A, int n, const double *__restrict__ b, const double *__restrict__ x,
                                                 double *__restrict__ r, double *part, Ctl *c, int force)
 {
     const VB vb = vb_grid();
@@ -2014,7 +2062,7 @@ __device__ __forceinline__ void b_rel_res(VB vb, M A, int n, const double *__res
 }
 
 template <class M>
-__global__ void __launch_bounds__(BS) k_rel_res(M A, int n, const double *__restrict__ b, const double *__restrict__ x,
+__global__ void PASS_BOUNDS(M, PASS_OTHER) k_rel_res(M A, int n, const double *__restrict__ b, const double *__restrict__ x,
                                                 float *__restrict__ r, double *part, Ctl *c, int force)
 {
     pdl_enter();
