@@ -480,7 +480,11 @@ __device__ __forceinline__ void dot_cols(const float *b, const CV<float, CW> &z,
 }
 
 // ------------------------------------------------------- V-cycle kernels --
-// The same passes as the single-vector cycle, on KB interleaved columns.
+// The same passes as the single-vector cycle, on KB interleaved columns.  The
+// launch bound of four blocks a SM of three of them lets the compiler keep more of
+// a thread's loads in flight (128^3, 8 columns: last post-smoothing step 92 -> 85 us,
+// CG product 88 -> 83, residual 42.5 -> 39.5); the interpolation loses by it (44 ->
+// 65), the others gain nothing.
 // DOT: the pass writes the CG's z and reduces (r, z) and (q, z) per column.
 
 // first two Chebyshev steps from zero: d0 = c0 dw b, r1 = b - A d0,
@@ -574,7 +578,7 @@ __global__ void __launch_bounds__(BS) kb_cheb0(M A, int n, const float *__restri
 // Chebyshev step k >= 2: r -= A d; dn = c1 d + c2 dw r; x += (add_prev ? d : 0) + dn;
 // the last step of an application (keep = 0, and DOT) stores neither r nor dn
 template <int KB, int CW, class M, bool DOT>
-__global__ void __launch_bounds__(BS) kb_chebk(M A, int n, const float *__restrict__ dw, float *__restrict__ r,
+__global__ void __launch_bounds__(BS, 4) kb_chebk(M A, int n, const float *__restrict__ dw, float *__restrict__ r,
                                                const float *__restrict__ d, float *__restrict__ dn, float *x,
                                                float *__restrict__ xo, float c1, float c2, int add_prev,
                                                int keep, const float *__restrict__ b0, const float *__restrict__ q,
@@ -653,7 +657,7 @@ __global__ void __launch_bounds__(BS) kb_axpy(long long m, const float *__restri
 
 // r = b - A x
 template <int KB, int CW, class M>
-__global__ void __launch_bounds__(BS) kb_residual(M A, int n, const float *__restrict__ b, const float *__restrict__ x,
+__global__ void __launch_bounds__(BS, 4) kb_residual(M A, int n, const float *__restrict__ b, const float *__restrict__ x,
                                                   float *__restrict__ r, const BlkCtl *c)
 {
     pdl_enter();
@@ -815,7 +819,7 @@ __global__ void __launch_bounds__(BS) kb_init(int n, const double *__restrict__ 
 // p_new = z + beta p_old (formed where gathered), q = A p_new, pq = (p_new, q),
 // alpha = rz / pq per column; a column at maxit stops here
 template <int KB, int CW, class M>
-__global__ void __launch_bounds__(BS) kb_dir_spmv(M A, int n, const float *__restrict__ z,
+__global__ void __launch_bounds__(BS, 4) kb_dir_spmv(M A, int n, const float *__restrict__ z,
                                                   const float *__restrict__ pold, float *__restrict__ pnew,
                                                   float *__restrict__ q, double *part, BlkCtl *c)
 {
