@@ -1180,18 +1180,37 @@ static void prolong_imp(Hier &H, const float *e, float *x, const Ctl *ctl, cudaS
     else launch_pdl(k_prolong_imp<1>, vgrid(H, I.n), st, P, e, x, ctl);
 }
 
-// x = Ainv b on the coarsest level (dense FP64 inverse), one warp per row
+// x = Ainv b on the coarsest level (dense FP64 inverse), COARSE_W warps per row.
+// FP64 issue bounds the product (a conversion and a multiply-add an entry), so its
+// few hundred rows have to reach every SM: with a warp a row the 369 rows of 128^3
+// were 47 blocks on 47 SMs.  128 x 128 x 1 solve 1.24 -> 1.21 ms, 128^3 8.70 -> 8.64
+// (to 1e-12); on eight interleaved columns it gained nothing.
+constexpr int COARSE_W = 4, COARSE_ROWS = BS / 32 / COARSE_W;
 template <class T>
 __device__ __forceinline__ void b_coarse(VB vb, int n, const double *__restrict__ Ainv, const T *__restrict__ b,
-                                               T *__restrict__ x, const Ctl *ctl) {
+                                         T *__restrict__ x, const Ctl *ctl)
+{
+    __shared__ double sh[BS / 32];
     if (finished(ctl)) return;
-    const int lane = threadIdx.x & 31;
-    for (int row = (vb.bid * BS + threadIdx.x) >> 5; row < n; row += (vb.nb * BS) >> 5) {
-        const double *a = Ainv + (size_t)row * n;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int row0 = vb.bid * COARSE_ROWS; row0 < n; row0 += vb.nb * COARSE_ROWS) {
+        const int row = row0 + w / COARSE_W;
         double s = 0.0;
-        for (int j = lane; j < n; j += 32) s += a[j] * (double)b[j];
+        if (row < n) {
+            const double *a = Ainv + (size_t)row * n;
+#pragma unroll 4
+            for (int j = (w % COARSE_W) * 32 + lane; j < n; j += 32 * COARSE_W) s += a[j] * (double)b[j];
+        }
         s = warp_sum(s);
-        if (lane == 0) x[row] = (T)s;
+        if (lane == 0) sh[w] = s;
+        __syncthreads();
+        if (lane == 0 && w % COARSE_W == 0 && row < n) {
+            double t = 0.0;
+#pragma unroll
+            for (int k = 0; k < COARSE_W; ++k) t += sh[w + k];
+            x[row] = (T)t;
+        }
+        __syncthreads();
     }
 }
 
@@ -1676,7 +1695,7 @@ static void vcycle_t(Hier &H, std::vector<CycLevel<T>> &C, const T *r, T *z, Ctl
     {
         CycLevel<T> &lc = C[L - 1];
         H.prof_bytes += vbytes(H, (double)lc.n * lc.n * 8.0 + 2.0 * lc.n * sx);
-        launch_pdl(k_coarse<T>, std::max(1, std::min(H.max_blocks, (lc.n * 32 + BS - 1) / BS)), st, lc.n, H.Ainv.p,
+        launch_pdl(k_coarse<T>, std::max(1, std::min(H.max_blocks, (lc.n + COARSE_ROWS - 1) / COARSE_ROWS)), st, lc.n, H.Ainv.p,
                    lc.b.p, lc.x.p, ctl);
     }
     for (int l = L - 2; l >= 0; --l) {

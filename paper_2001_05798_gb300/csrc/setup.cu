@@ -5,7 +5,7 @@
 // Stages per level: symmetrised strength of connection, distance-2 maximal
 // independent set by parallel rounds with hashed priorities, aggregation,
 // filtered matrix and Gershgorin bound, Jacobi-smoothed prolongator,
-// transpose, Galerkin product by a two-pass SpGEMM.  Then the dense inverse of
+// transpose, Galerkin product by SpGEMM.  Then the dense inverse of
 // the coarsest level and the conversion of every level to sliced ELL.
 //
 // Every floating-point operation that decides the hierarchy is an explicitly
