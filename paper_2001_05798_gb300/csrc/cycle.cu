@@ -593,8 +593,8 @@ struct MStenH {
 // at 128^3, CG product 17.2 -> 15.1, last post-smoothing step 17.3 -> 16.0, residual
 // 8.7 -> 6.7, first post-smoothing step 11.5 -> 11.0 (three blocks), pre-smoothing
 // 10.8 -> 12.7 (so none there).  One or two rows a thread: 117^3 solve 7.26 -> 6.75 ms;
-// FP64 at 96^3: stencil 10.2 -> 9.2, sliced ELL 9.2 -> 8.8 ms; BF16 and FP16
-// stencils 27.1 -> 26.9 ms at 256x256x128.  The FP32 sliced ELL lost (level 1 of
+// FP64 at 96^3: stencil 10.2 -> 9.2, sliced ELL 9.2 -> 8.8 ms; the BF16
+// stencil 27.1 -> 26.9 ms at 256x256x128 (the FP16 one lost).  The FP32 sliced ELL lost (level 1 of
 // 128^3 is 737 blocks: five a SM are one wave, four are two).
 enum { PASS_ZERO2, PASS_CHEB0, PASS_OTHER };
 template <class M>
@@ -615,10 +615,6 @@ struct MinBlocks<MSten<float, 1>> {
 };
 template <int R>
 struct MinBlocks<MStenB<R>> {
-    static constexpr int at(int) { return 1; }
-};
-template <int R>
-struct MinBlocks<MStenH<R>> {
     static constexpr int at(int) { return 1; }
 };
 template <int R>
