@@ -1239,6 +1239,16 @@ __device__ bool gj_invert_block(double &a, int i, int j, int bk)
     return true;
 }
 
+// *singular: 0, or 1 + the panel whose pivot block could not be inverted.  A
+// launch of panel K may set it to K + 2 for the next panel while its other
+// blocks read it, so only the value of an earlier launch, the same for every
+// thread, ends a block.
+__device__ __forceinline__ bool sweep_ended(const int *singular, int K)
+{
+    const int f = *(volatile const int *)singular;
+    return f != 0 && f <= K + 1;
+}
+
 // Q of the first panel (one block)
 __global__ void __launch_bounds__(256) k_sweep_pivot(int n, int bk, const double *__restrict__ M,
                                                      double *__restrict__ Q, int *__restrict__ singular)
@@ -1261,7 +1271,7 @@ __global__ void __launch_bounds__(256) k_sweep_panel(int n, int k0, int bk, cons
     __shared__ double c[GJB][GJB + 1], q[GJB][GJB + 1];
     const int i = threadIdx.x / GJB, j = threadIdx.x % GJB, row = blockIdx.x * GJB + i;
     gj_enter();
-    if (*(volatile const int *)singular) return;
+    if (sweep_ended(singular, k0 / GJB)) return;
     const double m = row < n && j < bk ? M[(size_t)row * n + k0 + j] : 0.0;
     c[i][j] = m;
     q[i][j] = Q[threadIdx.x];
@@ -1291,7 +1301,7 @@ __global__ void __launch_bounds__(256) k_sweep_update(int n, int k0, int bk, dou
     const int J = b - I * (I + 1) / 2;
     const double sg = neg ? -1.0 : 1.0;
     gj_enter();
-    if (*(volatile const int *)singular) return;
+    if (sweep_ended(singular, K)) return;
     const int r = I * GJB + i, s = J * GJB + j;
     double v;
     if (I == K && J == K) {
@@ -1323,7 +1333,7 @@ __global__ void __launch_bounds__(256) k_sweep_update(int n, int k0, int bk, dou
         const int bn = min(GJB, n - (K + 1) * GJB);
         double a = i < bn && j < bn ? v : (i == j ? 1.0 : 0.0);
         if (!gj_invert_block(a, i, j, bn)) {
-            if (threadIdx.x == 0) atomicExch(singular, 1);
+            if (threadIdx.x == 0) atomicExch(singular, K + 2);
             return;
         }
         Qn[threadIdx.x] = i < bn && j < bn ? a : 0.0;
