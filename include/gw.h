@@ -330,7 +330,9 @@ int gw_darcy_flux(const gw_grid *grid, const double *Kx, const double *Ky, const
                   const double *h, double *vx, double *vy, double *vz, void *stream);
 
 /* Applies one V-cycle z = M^-1 r (from a zero initial guess) with the
- * hierarchy's precision; r and z are n doubles on the device. */
+ * hierarchy's precision; r and z are n doubles on the device, at any address
+ * that is a multiple of 8 (FP64 form: one that is not a multiple of 16 costs a
+ * copy). */
 int gw_vcycle(gw_hierarchy H, const double *r, double *z, void *stream);
 
 /* Table-1 statistics: fills out[0..min(cap, levels)-1] and *nlevels. */

@@ -849,10 +849,24 @@ int gw_vcycle(gw_hierarchy H, const double *r, double *z, void *stream)
     if (!H || !r || !z) fail(GW_ERR_ARG, "gw_vcycle: null argument");
     if (H->h->batch) fail(GW_ERR_ARG, "gw_vcycle: the hierarchy's solve is in a batch");
     if (!is_device_ptr(r) || !is_device_ptr(z)) fail(GW_ERR_ARG, "gw_vcycle: r and z must be device pointers");
-    DeviceGuard g(H->h->dev);
+    Hier &hh = *H->h;
+    DeviceGuard g(hh.dev);
     cudaStream_t st = (cudaStream_t)stream;
     AllocStream alloc_scope(st);
-    vcycle_enqueue(*H->h, r, z, nullptr, false, st);
+    // The FP64 level-0 passes read r and write z 16 bytes at a time (the mixed
+    // form converts them double by double): a vector that starts elsewhere goes
+    // through the solver's own of the same length.
+    const size_t bytes = (size_t)hh.n * sizeof(double);
+    const bool f64 = hh.o.prec == GW_PREC_FP64;
+    const double *ra = r;
+    double *za = z;
+    if (f64 && (uintptr_t)r % 16) {
+        GW_CUDA(cudaMemcpyAsync(hh.r.p, r, bytes, cudaMemcpyDeviceToDevice, st));
+        ra = hh.r.p;
+    }
+    if (f64 && (uintptr_t)z % 16) za = hh.z.p;
+    vcycle_enqueue(hh, ra, za, nullptr, false, st);
+    if (za != z) GW_CUDA(cudaMemcpyAsync(z, za, bytes, cudaMemcpyDeviceToDevice, st));
     GW_CUDA(cudaStreamSynchronize(st));
     GW_API_END
 }
