@@ -233,7 +233,11 @@ int gw_matrix_export(gw_matrix A, int *rowptr, int *col, double *val, void *stre
  * adds index validation of every level after the setup (GW_ERR_SETUP on a
  * bad index); GW_SETUP_FORMS=thread|warp forces one of the two row-parallel
  * forms of the SpGEMM and prolongator passes (the library otherwise picks
- * one per product; both give the same bits).
+ * one per product; both give the same bits); GW_SPGEMM_TEMP=bytes limits the
+ * temporary of a product (4 GB; past it, or where the device has no room for
+ * it, the product takes two runs and no temporary, with the same bits);
+ * GW_ALLOC_REFUSE=min,max,count refuses the first count device allocations
+ * of min to max bytes.
  *   A     assembled matrix; the hierarchy keeps a reference to it (freeing A
  *         before H is the caller's error).
  *   opts  host struct or NULL for the defaults.

@@ -1050,10 +1050,17 @@ __global__ void k_sg_numeric(int nr, const int *__restrict__ rows, const int *__
     }
 }
 
-#ifndef GW_SGG_TEMP_MAX
-#define GW_SGG_TEMP_MAX (4.0 * (1 << 30))
-#endif
-constexpr double SGG_TEMP_MAX = GW_SGG_TEMP_MAX;
+// Bytes that the temporary of a product by lane groups may take (the product
+// takes two runs instead beyond it): 4 GB, or GW_SPGEMM_TEMP in the
+// environment, read once, so that tests can check the two-run form.
+static double spgemm_temp_max()
+{
+    static const double b = [] {
+        const char *e = getenv("GW_SPGEMM_TEMP");
+        return e && *e ? atof(e) : 4.0 * (1 << 30);
+    }();
+    return b;
+}
 
 // the temporary's rows to their places; rows of more than cap entries are the
 // warp kernels'
@@ -1086,11 +1093,20 @@ void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
     // column on the fine levels) and the mean row length of Rm.  The warp form
     // keeps products whose rows would mostly pass 128 columns.  Up to 4 GB of
     // temporary (22 million fine cells) one run and a packing pass, 20 % of the
-    // run; beyond, two runs.
+    // run; beyond, or where the device has no room for the temporary, or for the
+    // product beside it, two runs.  With the temporary a setup at 160^3 takes 16.7
+    // ms and at most 524 bytes a cell (mixed; FP64 549), with two runs 19.7 ms and
+    // 451 (549).
     const double m = (double)Rm.nnz / std::max(1, Rm.nr), per_row = L.nr ? (double)L.nnz / L.nr * m : 0.0;
     const int cap = per_row <= 40.0 ? 16 : per_row <= 1000.0 ? 64 : 128;
     const bool groups = setup_forms() ? setup_forms() == 1 : per_row <= 16384.0;
-    const bool temp = (double)L.nr * cap * 12.0 <= SGG_TEMP_MAX;
+    bool temp = groups && (double)L.nr * cap * 12.0 <= spgemm_temp_max();
+    auto no_temp = [&](const Error &e) {
+        if (e.code != GW_ERR_OOM || !temp) throw;
+        tci.release();
+        tcv.release();
+        temp = false;
+    };
     auto run_groups = [&](const int *crp, int *cnt, int *oci, double *ov) {
         auto run = [&](auto kernel, int G, size_t smem) {
             // always the same value per kernel (see below)
@@ -1110,8 +1126,12 @@ void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
     if (groups) {
         long_rows.alloc((size_t)L.nr);
         if (temp) {
-            tci.alloc((size_t)L.nr * cap);
-            tcv.alloc((size_t)L.nr * cap);
+            try {
+                tci.alloc((size_t)L.nr * cap);
+                tcv.alloc((size_t)L.nr * cap);
+            } catch (const Error &e) {
+                no_temp(e);
+            }
         }
         run_groups(nullptr, C.rp.p, tci.p, tcv.p);
         nlong = read_int(ctr.p, st);
@@ -1152,8 +1172,14 @@ void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st)
     }
     exclusive_scan(C.rp.p, C.rp.p, C.nr, st);
     C.nnz = read_int(C.rp.p + C.nr, st);
-    C.ci.alloc((size_t)C.nnz);
-    C.v.alloc((size_t)C.nnz);
+    try {
+        C.ci.alloc((size_t)C.nnz);
+        C.v.alloc((size_t)C.nnz);
+    } catch (const Error &e) {
+        no_temp(e);
+        C.ci.alloc((size_t)C.nnz);
+        C.v.alloc((size_t)C.nnz);
+    }
     if (groups && !temp) {
         run_groups(C.rp.p, nullptr, C.ci.p, C.v.p);
     } else if (groups && nlong < L.nr) {

@@ -1,5 +1,6 @@
 // util.cu -- error plumbing, device scan and small host helpers of libgw.
 #include <stdarg.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <atomic>
@@ -84,16 +85,36 @@ static int current_pool_device()
     return dev;
 }
 
+// GW_ALLOC_REFUSE=min,max,count in the environment (read once, for tests): the
+// first count allocations of min to max bytes are refused as if the device
+// were full.
+static bool refused(size_t bytes)
+{
+    static unsigned long long lo = 0, hi = 0;
+    static std::atomic<long long> left{[] {
+        long long n = 0;
+        const char *e = getenv("GW_ALLOC_REFUSE");
+        return e && sscanf(e, "%llu,%llu,%lld", &lo, &hi, &n) == 3 ? n : 0LL;
+    }()};
+    return left.load() > 0 && bytes >= lo && bytes <= hi && left.fetch_sub(1) > 0;
+}
+
 cudaError_t dev_malloc(void **p, size_t bytes, int *pool_dev)
 {
     std::unique_lock<std::mutex> lk(g_alloc_mu);
     g_alloc_cv.wait(lk, [] { return g_captures == 0; });
     g_device_allocs.fetch_add(1);
     *pool_dev = -1;
+    if (refused(bytes)) return cudaErrorMemoryAllocation;
     const int dev = t_alloc_on ? current_pool_device() : -1;
-    if (dev < 0) return cudaMalloc(p, bytes);
-    const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool_of(dev).pool, t_alloc_stream);
-    if (e == cudaSuccess) *pool_dev = dev;
+    cudaError_t e;
+    if (dev < 0) {
+        e = cudaMalloc(p, bytes);
+    } else {
+        e = cudaMallocFromPoolAsync(p, bytes, pool_of(dev).pool, t_alloc_stream);
+        if (e == cudaSuccess) *pool_dev = dev;
+    }
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // the caller's: not the next launch check's
     return e;
 }
 
