@@ -70,12 +70,12 @@ Hier::~Hier()
     if (ctl_host) host_free(ctl_host);
 }
 
-// the smoother's weights: scale / a_ii, or the given inverse diagonal (scale 1)
-__global__ void k_make_dw(int n, const double *__restrict__ d, const double *__restrict__ inv, double scale,
-                          float *__restrict__ of, double *__restrict__ od)
+// the smoother's weights: scale / a_ii (Jacobi) or 1 / a_ii (Chebyshev, d already inverse)
+__global__ void k_make_dw(int n, const double *__restrict__ d, int inverse, double scale, float *__restrict__ of,
+                          double *__restrict__ od)
 {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const double w = inv ? inv[i] : scale / d[i];
+        const double w = inverse ? d[i] : scale / d[i];
         if (of) of[i] = (float)w;
         if (od) od[i] = w;
     }
@@ -124,27 +124,27 @@ static long long store_level(Hier &H, int k, const DCSR &A, const DCSR *P, const
     const bool f64 = o.prec == GW_PREC_FP64;
     const int n = A.nr;
     long long bytes = 0;
-    DBuf<double> diag, inv;
-    const double rhoJ = setup_gershgorin(A, diag, inv, st);
+    const bool cheb = o.smoother != GW_SMOOTH_JACOBI;
+    DBuf<double> diag;  // Chebyshev: its inverse
+    const double rhoJ = setup_gershgorin(A, diag, cheb, st);
     H.info[(size_t)k].jacobi_w = (4.0 / 3.0) / rhoJ;
     double scale = 1.0;
     double c0 = 0.0, c1[8] = {0}, c2[8] = {0};
-    if (o.smoother == GW_SMOOTH_JACOBI) {
+    if (!cheb) {
         scale = H.info[(size_t)k].jacobi_w;
     } else {
-        const double lam = setup_power_lambda(A, inv.p, o.seed, k, st);
+        const double lam = setup_power_lambda(A, diag.p, o.seed, k, st);
         H.info[(size_t)k].lambda_max = lam;
         cheb_coeffs(lam, o.degree, c0, c1, c2);
     }
     const int g = (int)std::min<long long>(((long long)n + 255) / 256, 152LL * 16);
-    const double *dinv = o.smoother == GW_SMOOTH_JACOBI ? nullptr : inv.p;
     if (f64) {
         CycLevel<double> &c = H.cd[(size_t)k];
         to_store<double>(A, c.A, k == 0 ? FMT_STEN : choose_fmt(A), H.gnx, H.gny, H.gnz, st);
         if (P) to_store<double>(*P, c.P, choose_fmt(*P), 0, 0, 0, st);
         if (R) to_store<double>(*R, c.R, sorted_sell(choose_fmt(*R)), 0, 0, 0, st);
         c.dw.alloc((size_t)n);
-        gw_launch(k_make_dw, std::max(g, 1), 256, 0, st, n, diag.p, dinv, scale, nullptr, c.dw.p);
+        gw_launch(k_make_dw, std::max(g, 1), 256, 0, st, n, diag.p, cheb ? 1 : 0, scale, nullptr, c.dw.p);
         c.c0 = c0;
         memcpy(c.c1, c1, sizeof c1);
         memcpy(c.c2, c2, sizeof c2);
@@ -167,7 +167,7 @@ static long long store_level(Hier &H, int k, const DCSR &A, const DCSR *P, const
         if (k == 0 && H.p0.n) bytes += (long long)H.p0.bytes();
         if (R) to_store<float>(*R, c.R, sorted_sell(choose_fmt(*R)), 0, 0, 0, st);
         c.dw.alloc((size_t)n);
-        gw_launch(k_make_dw, std::max(g, 1), 256, 0, st, n, diag.p, dinv, scale, c.dw.p, nullptr);
+        gw_launch(k_make_dw, std::max(g, 1), 256, 0, st, n, diag.p, cheb ? 1 : 0, scale, c.dw.p, nullptr);
         c.c0 = c0;
         memcpy(c.c1, c1, sizeof c1);
         memcpy(c.c2, c2, sizeof c2);

@@ -342,8 +342,8 @@ bool setup_implicit_p(const DCSR &A, const unsigned char *S, const int *agg, int
                       int nz, ImplP &out, cudaStream_t st);
 void setup_spgemm(const DCSR &L, const DCSR &Rm, DCSR &C, cudaStream_t st);
 void setup_dense_inverse(const DCSR &A, DBuf<double> &Ainv, cudaStream_t st);
-// max_i sum|a_ij|/a_ii; the diagonal and its inverse
-double setup_gershgorin(const DCSR &A, DBuf<double> &diag, DBuf<double> &inv, cudaStream_t st);
+// max_i sum|a_ij|/a_ii; the diagonal or its inverse
+double setup_gershgorin(const DCSR &A, DBuf<double> &diag, bool inverse, cudaStream_t st);
 double setup_power_lambda(const DCSR &A, const double *inv, uint64_t seed, int level, cudaStream_t st);
 
 template <class T>

@@ -1402,11 +1402,10 @@ void setup_dense_inverse(const DCSR &A, DBuf<double> &Ainv, cudaStream_t st)
 }
 
 // ------------------------------------------------- smoother data (per level) --
-// diagonal, its inverse (for the power iteration and the smoother's weights),
-// and the largest Gershgorin ratio
+// the diagonal, or its inverse (for the power iteration and the Chebyshev
+// weights; an FP64 division a row), and the largest Gershgorin ratio
 __global__ void k_gersh(int n, const int *__restrict__ rp, const int *__restrict__ ci, const double *__restrict__ v,
-                        double *__restrict__ d, double *__restrict__ inv,
-                        unsigned long long *__restrict__ rho_bits)
+                        double *__restrict__ d, int inverse, unsigned long long *__restrict__ rho_bits)
 {
     unsigned long long best = 0;
     GRID_STRIDE(ii, n)
@@ -1417,8 +1416,7 @@ __global__ void k_gersh(int n, const int *__restrict__ rp, const int *__restrict
             s += fabs(v[e]);
             if (ci[e] == i) dd = v[e];
         }
-        d[i] = dd;
-        inv[i] = 1.0 / dd;
+        d[i] = inverse ? 1.0 / dd : dd;
         const double ratio = s / dd;
         if (ratio > 0.0 && isfinite(ratio)) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(ratio);
@@ -1428,13 +1426,12 @@ __global__ void k_gersh(int n, const int *__restrict__ rp, const int *__restrict
     block_atomic_max(best, rho_bits);
 }
 
-double setup_gershgorin(const DCSR &A, DBuf<double> &diag, DBuf<double> &inv, cudaStream_t st)
+double setup_gershgorin(const DCSR &A, DBuf<double> &diag, bool inverse, cudaStream_t st)
 {
     diag.alloc((size_t)A.nr);
-    inv.alloc((size_t)A.nr);
     DBuf<unsigned long long> rb(1);
     GW_CUDA(cudaMemsetAsync(rb.p, 0, sizeof(unsigned long long), st));
-    gw_launch(k_gersh, nblk(A.nr, 256), 256, 0, st, A.nr, A.rp.p, A.ci.p, A.v.p, diag.p, inv.p, rb.p);
+    gw_launch(k_gersh, nblk(A.nr, 256), 256, 0, st, A.nr, A.rp.p, A.ci.p, A.v.p, diag.p, inverse ? 1 : 0, rb.p);
     GW_LAUNCH_CHECK();
     unsigned long long bits = 0;
     GW_CUDA(cudaMemcpyAsync(&bits, rb.p, sizeof bits, cudaMemcpyDeviceToHost, st));
