@@ -1558,10 +1558,12 @@ static void smooth(Hier &H, std::vector<CycLevel<T>> &C, int l, const T *b, bool
                 const bool f2 = fin && m == 2;
                 const int keep = m > 2;
                 timed(H, kind(), st, [&] {
-                    H.prof_bytes += vbytes(H, amat + 2.0 * dn * sx + (keep ? 3.0 : 1.0) * dn * sx +
-                                                  (f2 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
                     // d0 in d2, stored by the restriction on the coarser levels
                     constexpr bool PRE = sizeof(T) == 8;
+                    // with PRE d0 is read too, and on level 0 dw and b read and d0 written before
+                    H.prof_bytes += vbytes(H, amat + 2.0 * dn * sx + (keep ? 3.0 : 1.0) * dn * sx +
+                                                  (PRE ? (l == 0 ? 4.0 : 1.0) * dn * sx : 0.0) +
+                                                  (f2 ? dn * sx * (q ? 2.0 : 1.0) : 0.0));
                     const T *d0 = PRE ? lv.d2.p : nullptr;
                     if (PRE && l == 0) {
                         if (n % 2 == 0) launch_pdl(k_first<T, 2>, vgrid(H, n / 2), st, n, lv.dw.p, b, lv.d2.p, (T)lv.c0, ctl);
@@ -1673,7 +1675,9 @@ static void vcycle_t(Hier &H, std::vector<CycLevel<T>> &C, const T *r, T *z, Ctl
                     return;
                 }
             }
-            H.prof_bytes += vbytes(H, mat_bytes(lv.R) + dn * sx + (double)lv.R.nr * sx);
+            // d0 of the next level stored (FP64): dw read, d0 written
+            const double nd0 = sizeof(T) == 8 && first.d0 ? 2.0 : 0.0;
+            H.prof_bytes += vbytes(H, mat_bytes(lv.R) + dn * sx + (1.0 + nd0) * (double)lv.R.nr * sx);
             with_mat(lv.R, [&](auto Rm) {
                 using M = decltype(Rm);
                 if constexpr (M::R == 1)
