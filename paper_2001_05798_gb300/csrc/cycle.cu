@@ -2714,7 +2714,7 @@ static int pass_nb(const BSlot &S, const BLaunch &c)
     case BP_RESTRICT_U:
     case BP_PROLONG_IMP: return bnb(n0 / S.p0r);
     case BP_RESTRICT_SUM: return bnb(4LL * S.nc0);
-    case BP_COARSE: return bnb(32LL * S.lv[c.level].n);
+    case BP_COARSE: return bnb((long long)(BS / COARSE_ROWS) * S.lv[c.level].n);
     case BP_SPMV: return bnb(bmat_threads(S.lv[c.level].R, S.lv[c.level].R.nr));
     case BP_PROLONG: return bnb(bmat_threads(S.lv[c.level].P, S.lv[c.level].n));
     default: return bnb(bmat_threads(S.lv[c.level].A, S.lv[c.level].n));
