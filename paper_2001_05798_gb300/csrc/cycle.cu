@@ -2440,9 +2440,9 @@ int pcg_run(Hier &H, double tol, int maxit, int *iters, double *relres, cudaStre
 // passes (the CG product and update, the reliable update, and the V-cycle's
 // passes level by level, padded to the deepest hierarchy); each pass is one
 // launch whose work list holds (slot, virtual block) items for every slot
-// that has that pass.  A slot's passes use a virtual grid fixed by its own
-// size, and its reductions use its own partial-sum array and counters, so a
-// solve gives the same bits alone and in any mix.  The iteration is captured
+// that has that pass.  A slot's passes with a dot product use a virtual grid
+// fixed by its own size, and its reductions its own partial-sum array and
+// counters, so a solve gives the same bits alone and in any mix.  The iteration is captured
 // once as a CUDA graph and replayed; admission and removal of slots between
 // replays only rewrite the device slot table and work lists.  Slots finish
 // independently: a finished slot's passes return at once until it is taken.
@@ -2450,10 +2450,15 @@ int pcg_run(Hier &H, double tol, int maxit, int *iters, double *relres, cudaStre
 constexpr int BATCH_MAXL = 12;   // levels of a hierarchy in a batch
 // Virtual blocks of one pass of one slot.  A work item costs a few microseconds
 // whatever its rows (slot table, descriptor and first loads one after the other,
-// a reduction's barriers), so a slot has no more of them than two a SM.  Against
-// 1024 (ms a set of solves to 1e-12): eight of sides 33-96 18.6 -> 16.4, 45 and
-// 57 4.6 -> 3.9, one of 96 6.4 -> 6.0, four of 160 59.2 -> 56.1; 152 loses on few
-// larger solves (one of 96 7.5), 608 gains less.
+// a reduction's barriers), so that a slot has no more of them than two a SM, half
+// of the kernels' resident blocks: two slots fill one wave.  A pass without a dot
+// product lets a slot that is alone in it have the whole wave (pass_cap).
+// ms a set of solves to 1e-12, by cap 1024 | 608 | 304 | 304 and the wave alone:
+// one of 117 - | - | 10.97 | 9.20, of 128 10.7 | 10.2 | 11.2 | 10.1, of 160 18.0 |
+// 17.0 | 21.0 | 17.0; two of 96 9.9 | 9.9 | 8.5 | 8.5, of 160 31.9 | 29.2 | 27.7 | 27.0;
+// four of 160 55.1 | 54.0 | 50.1 | 50.1; eight of 33-96 16.1 | 15.5 | 14.3 | 14.2.
+// Cutting every slot's items to one wave in all lost on eight (20.3: items of the
+// 4-row and 1-row stencils differ in cost); a cap of 456 loses on pairs (9.6, 30.5).
 constexpr int BATCH_NB_CAP = 304;
 
 enum { BM_NONE = 0, BM_STEN4, BM_STEN2, BM_STEN1, BM_SELL, BM_CSR32 };
@@ -2641,6 +2646,7 @@ struct Batch {
     std::vector<int> state;           // 0 free, 1 running, 2 finished (not yet taken)
     std::vector<BSlot> hslots;        // host image of the slot table
     std::vector<BLaunch> launches;    // the iteration's pass sequence for lmax levels
+    std::vector<int> wave;            // and the resident blocks of each pass's kernel
     DBuf<BSlot> dslots;
     DBuf<int4> work;
     DBuf<int> wcnt;                   // per launch: offset and count of its items
@@ -2692,8 +2698,8 @@ static BMat bmat_of(const MatStore<float> &M)
     return b;
 }
 
-// virtual blocks of one pass of one slot (a function of the slot alone)
-static int bnb(long long threads) { return (int)std::max(1LL, std::min<long long>((threads + BS - 1) / BS, BATCH_NB_CAP)); }
+// blocks that `threads` work items ask for
+static int bnb(long long threads) { return (int)std::max(1LL, (threads + BS - 1) / BS); }
 
 static int bmat_rows_per_thread(const BMat &m) { return m.fmt == BM_STEN4 ? 4 : m.fmt == BM_STEN2 ? 2 : 1; }
 
@@ -2703,7 +2709,8 @@ static long long bmat_threads(const BMat &m, int n)
     return (n + bmat_rows_per_thread(m) - 1) / bmat_rows_per_thread(m);
 }
 
-static int pass_nb(const BSlot &S, const BLaunch &c)
+// blocks that one pass of one slot asks for
+static int pass_blocks(const BSlot &S, const BLaunch &c)
 {
     const int n0 = S.lv[0].n;
     switch (c.kind) {
@@ -2772,34 +2779,44 @@ static std::vector<BLaunch> batch_sequence(int lmax, int m)
     return q;
 }
 
-template <int KIND>
-static void kb_launch(Batch &B, int idx, cudaStream_t s)
+using KbPass = void (*)(const BSlot *, const int4 *, const int *, int, BLaunch);
+static KbPass kb_kernel(int kind)
 {
-    launch_pdl(kb_pass<KIND>, kernel_wave((const void *)kb_pass<KIND>, BS), s, (const BSlot *)B.dslots.p,
-               (const int4 *)B.work.p, (const int *)B.wcnt.p, idx, B.launches[(size_t)idx]);
+    switch (kind) {
+    case BP_DIR_SPMV: return kb_pass<BP_DIR_SPMV>;
+    case BP_UPDATE: return kb_pass<BP_UPDATE>;
+    case BP_REL_FOLD: return kb_pass<BP_REL_FOLD>;
+    case BP_REL_RES: return kb_pass<BP_REL_RES>;
+    case BP_ZERO2: return kb_pass<BP_ZERO2>;
+    case BP_CHEBK: return kb_pass<BP_CHEBK>;
+    case BP_RESID: return kb_pass<BP_RESID>;
+    case BP_RESTRICT_U: return kb_pass<BP_RESTRICT_U>;
+    case BP_RESTRICT_SUM: return kb_pass<BP_RESTRICT_SUM>;
+    case BP_SPMV: return kb_pass<BP_SPMV>;
+    case BP_COARSE: return kb_pass<BP_COARSE>;
+    case BP_PROLONG: return kb_pass<BP_PROLONG>;
+    case BP_PROLONG_IMP: return kb_pass<BP_PROLONG_IMP>;
+    case BP_CHEB0: return kb_pass<BP_CHEB0>;
+    default: return kb_pass<BP_CHEBK_DOT>;
+    }
+}
+
+// Virtual blocks at most of one pass of one slot, of `parts` slots in the pass.
+// The blocks of a pass with a dot product decide the order of its sums, so
+// there the cap depends on nothing else; the others give the same bits on any
+// number of blocks, and a slot may take its share of the wave.
+static int pass_cap(int kind, int wave, int parts)
+{
+    const bool reduces = kind == BP_DIR_SPMV || kind == BP_UPDATE || kind == BP_REL_RES || kind == BP_CHEBK_DOT;
+    return reduces ? BATCH_NB_CAP : std::max(BATCH_NB_CAP, wave / std::max(1, parts));
 }
 
 static void batch_enqueue_iteration(Batch &B, cudaStream_t s)
 {
     for (int i = 0; i < (int)B.launches.size(); ++i) {
-        switch (B.launches[(size_t)i].kind) {
-        case BP_DIR_SPMV: kb_launch<BP_DIR_SPMV>(B, i, s); break;
-        case BP_UPDATE: kb_launch<BP_UPDATE>(B, i, s); break;
-        case BP_REL_FOLD: kb_launch<BP_REL_FOLD>(B, i, s); break;
-        case BP_REL_RES: kb_launch<BP_REL_RES>(B, i, s); break;
-        case BP_ZERO2: kb_launch<BP_ZERO2>(B, i, s); break;
-        case BP_CHEBK: kb_launch<BP_CHEBK>(B, i, s); break;
-        case BP_RESID: kb_launch<BP_RESID>(B, i, s); break;
-        case BP_RESTRICT_U: kb_launch<BP_RESTRICT_U>(B, i, s); break;
-        case BP_RESTRICT_SUM: kb_launch<BP_RESTRICT_SUM>(B, i, s); break;
-        case BP_SPMV: kb_launch<BP_SPMV>(B, i, s); break;
-        case BP_COARSE: kb_launch<BP_COARSE>(B, i, s); break;
-        case BP_PROLONG: kb_launch<BP_PROLONG>(B, i, s); break;
-        case BP_PROLONG_IMP: kb_launch<BP_PROLONG_IMP>(B, i, s); break;
-        case BP_CHEB0: kb_launch<BP_CHEB0>(B, i, s); break;
-        case BP_CHEBK_DOT: kb_launch<BP_CHEBK_DOT>(B, i, s); break;
-        default: break;
-        }
+        const BLaunch &c = B.launches[(size_t)i];
+        launch_pdl(kb_kernel(c.kind), B.wave[(size_t)i], s, (const BSlot *)B.dslots.p, (const int4 *)B.work.p,
+                   (const int *)B.wcnt.p, i, c);
     }
     launch_pdl(kb_summary, 1, s, (const BSlot *)B.dslots.p, B.max_slots, B.dsum.p);
     GW_CUDA(cudaMemcpyAsync(B.hsum, B.dsum.p, sizeof(BSum) * (size_t)B.max_slots, cudaMemcpyDeviceToHost, s));
@@ -2810,18 +2827,18 @@ static void batch_enqueue_iteration(Batch &B, cudaStream_t s)
 static void batch_rebuild_work(Batch &B)
 {
     const int nl = (int)B.launches.size();
-    size_t total = 0;
-    for (int i = 0; i < nl; ++i)
-        for (int s = 0; s < B.max_slots; ++s)
-            if (pass_has(B.hslots[(size_t)s], B.launches[(size_t)i])) total += (size_t)pass_nb(B.hslots[(size_t)s], B.launches[(size_t)i]);
-    if (total > B.work_cap) fail(GW_ERR_OOM, "batch: work lists exceed their capacity");
     size_t k = 0;
     for (int i = 0; i < nl; ++i) {
+        const BLaunch &c = B.launches[(size_t)i];
+        int parts = 0;
+        for (const BSlot &S : B.hslots) parts += pass_has(S, c);
+        const int cap = pass_cap(c.kind, B.wave[(size_t)i], parts);
         B.hwcnt[2 * i] = (int)k;
         for (int s = 0; s < B.max_slots; ++s) {
             const BSlot &S = B.hslots[(size_t)s];
-            if (!pass_has(S, B.launches[(size_t)i])) continue;
-            const int nb = pass_nb(S, B.launches[(size_t)i]);
+            if (!pass_has(S, c)) continue;
+            const int nb = std::min(pass_blocks(S, c), cap);
+            if (k + (size_t)nb > B.work_cap) fail(GW_ERR_OOM, "batch: work lists exceed their capacity");
             for (int v = 0; v < nb; ++v) B.hwork[k++] = make_int4(s, v, nb, 0);
         }
         B.hwcnt[2 * i + 1] = (int)(k - (size_t)B.hwcnt[2 * i]);
@@ -2839,7 +2856,12 @@ static void batch_capture(Batch &B, int lmax)
     const size_t nl = seq.size();
     // launch table and work-list capacity for this sequence
     DBuf<int> wcnt(2 * nl);
-    size_t cap = nl * (size_t)B.max_slots * BATCH_NB_CAP;
+    size_t cap = 0;
+    std::vector<int> wave;
+    for (const BLaunch &c : seq) {
+        wave.push_back(kernel_wave((const void *)kb_kernel(c.kind), BS));
+        cap += (size_t)std::max(B.max_slots * BATCH_NB_CAP, pass_cap(c.kind, wave.back(), 1));
+    }
     DBuf<int4> work(cap);
     int *hw = nullptr;
     int4 *hk = nullptr;
@@ -2853,6 +2875,7 @@ static void batch_capture(Batch &B, int lmax)
     B.work = std::move(work);
     B.work_cap = cap;
     B.launches = seq;
+    B.wave = std::move(wave);
     if (B.g) cudaGraphExecDestroy(B.g);
     B.g = nullptr;
     for (int i = 0; i < (int)nl; ++i) {  // kernels are loaded outside the capture
