@@ -66,7 +66,9 @@ typedef struct {
 } gw_bc;
 
 /* Arithmetic of the solve.  The coarsest level always uses the FP64 dense
- * inverse and dot products are always summed in FP64 across threads.
+ * inverse.  Dot products of FP64 vectors are summed in FP64, those of FP32
+ * vectors as error-free FP32 pairs a thread and in three FP32 words (about 70
+ * bits; in FP64 from 2^100 on) across threads.
  * GW_PREC_FP64: the hierarchy, the V-cycle and every CG vector in FP64.
  * GW_PREC_MIXED32: the hierarchy and V-cycle in FP32, the CG recurrence in
  * FP32 against the FP32 level-0 operator, and the solution in FP64 by

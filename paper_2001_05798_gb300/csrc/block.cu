@@ -483,8 +483,8 @@ __device__ __forceinline__ void dot_cols(const float *b, const CV<float, CW> &z,
 // The same passes as the single-vector cycle, on KB interleaved columns.  The
 // launch bound of four blocks a SM of three of them lets the compiler keep more of
 // a thread's loads in flight (128^3, 8 columns: last post-smoothing step 92 -> 85 us,
-// CG product 88 -> 83, residual 42.5 -> 39.5); the interpolation loses by it (44 ->
-// 65), the others gain nothing.
+// CG product 88 -> 83, residual 42.5 -> 39.5, times not overlapped by the kernels
+// before); the interpolation loses by it (44 -> 65), the others gain nothing.
 // DOT: the pass writes the CG's z and reduces (r, z) and (q, z) per column.
 
 // first two Chebyshev steps from zero: d0 = c0 dw b, r1 = b - A d0,

@@ -589,13 +589,15 @@ struct MStenH {
 // without the bound ptxas keeps the registers low (32-62, 4-8 blocks) by issuing a
 // thread's loads late; asked for few blocks it keeps the loads of both unrolled
 // row groups, or of all neighbours, in flight, which hides more than the blocks
-// lost.  Measured per pass (us, without -> with): FP32 stencil of 4 rows a thread
-// at 128^3, CG product 17.2 -> 15.1, last post-smoothing step 17.3 -> 16.0, residual
-// 8.7 -> 6.7, first post-smoothing step 11.5 -> 11.0 (three blocks), pre-smoothing
-// 10.8 -> 12.7 (so none there).  One or two rows a thread: 117^3 solve 7.26 -> 6.75 ms;
-// FP64 at 96^3: stencil 10.2 -> 9.2, sliced ELL 9.2 -> 8.8 ms; the BF16
-// stencil 27.1 -> 26.9 ms at 256x256x128 (the FP16 one lost).  The FP32 sliced ELL lost (level 1 of
-// 128^3 is 737 blocks: five a SM are one wave, four are two).
+// lost.  Without -> with, events around each launch of a profiled solve (us) and
+// whole solves to 1e-12 (ms).  FP32 stencil of 4 rows a thread, 128^3: CG product
+// 21.0 -> 19.0, residual 12.8 -> 11.2, last post-smoothing step 21.9 -> 20.1, first
+// one 16.7 either way (three blocks; two lost), pre-smoothing lost with any; solve 7.17 ->
+// 6.86.  One or two rows a thread: 117^3 solve 6.84 -> 6.40.  FP64 at 96^3, stencil and
+// sliced ELL: 9.74 -> 8.43.  BF16 stencil: 117^3 6.76 -> 6.45, 118^3 6.21 -> 6.04,
+// 256x256x128 23.05 -> 22.96 (the FP16 one lost).  FP32 sliced ELL: with four blocks
+// solves of 96, 117 and 144 cubed gain 1-2 %, of 128 and 160 cubed lose 5 and 3 %; with five
+// all lose 1-3 %; so none there.
 enum { PASS_ZERO2, PASS_CHEB0, PASS_OTHER };
 template <class M>
 struct MinBlocks {
@@ -877,7 +879,8 @@ __global__ void PASS_BOUNDS(M, PASS_OTHER) k_residual(M A, int n, const BT *__re
 // writes to, d0 = c0 dw b, stored beside b (d0 null: not needed).  FP64 issue
 // bounds that level's pre-smoothing, and forming d0 from dw and b at every
 // entry cost two FP64 multiplications (and a gather) more an entry: at 96^3 the
-// level-1 pass took 44 us, 22 with the stored d0.  The FP32 form keeps forming it
+// level-1 pass took 44 us, 22 with the stored d0 (time not overlapped by the
+// kernels before it, here and below).  The FP32 form keeps forming it
 // where gathered: its level-1 pass is bound by fetching the matrix (15.9 against
 // 15.0 us at 128^3, and the restriction paid 1 us for the store).
 template <class T>
@@ -1150,7 +1153,7 @@ __device__ __forceinline__ void b_restrict_sum(VB vb, int nc, const int *__restr
     }
 }
 
-__global__ void __launch_bounds__(BS, 2) k_restrict_sum(int nc, const int *__restrict__ mptr, const int *__restrict__ mem,
+__global__ void __launch_bounds__(BS) k_restrict_sum(int nc, const int *__restrict__ mptr, const int *__restrict__ mem,
                                                      const float *__restrict__ u, float *__restrict__ rc,
                                                      const Ctl *ctl)
 {
@@ -1359,7 +1362,7 @@ __global__ void PASS_BOUNDS(M, PASS_OTHER) k_chebk(M A, int n, const typename M:
 // follow (keep).  DOT: x is the CG's z and (b, z), (q, z) are reduced.
 // PRE in the FP64 form: the restriction stores d0 on the coarser levels, a pass
 // of its own (k_first) on level 0, where the pre-smoothing so went from 54 us to
-// 27 + 7 at 96^3.
+// 27 + 7 at 96^3 (time not overlapped by the kernels before it).
 template <class M, class OT, bool DOT, bool PRE>
 __device__ __forceinline__ void b_cheb_zero2(VB vb, M A, int n, const typename M::value_type *__restrict__ dw,
                                                    const typename M::value_type *__restrict__ b,
@@ -1755,7 +1758,7 @@ void vcycle_enqueue(Hier &H, const double *r, double *z, Ctl *ctl, bool dot, cud
 // Two forms share these kernels.  FP64: every vector and the matrix of the
 // CG recurrence in FP64.  Mixed: the CG recurrence (p, q, r, z and the
 // correction xs) runs in FP32 against the FP32 level-0 operator, dot
-// products are summed in FP64 across threads, and the solution is kept in
+// products are summed as the notes of kern.cuh say, and the solution is kept in
 // FP64 by reliable updates (van der Vorst & Ye 2000): whenever the recursive
 // residual has dropped by the factor delta since the last update, or passes
 // the stopping test, xs is folded into the FP64 solution and the residual is
@@ -1914,7 +1917,7 @@ __device__ __forceinline__ void b_cg_update(VB vb, int n, V *__restrict__ x, V *
     // two of the thread's row groups per step, all their loads issued first
     // (the second group's loads no longer wait for the first's); the groups
     // are added to the dot in the same order as one at a time.  The launch bound
-    // of two blocks lets the compiler hold them all (128^3: 12.8 -> 11.0 us)
+    // of two blocks lets the compiler hold them all (128^3: 16.7 -> 15.0 us by events)
     const int stride = R * vb.nb * BS;
     for (int i = R * (vb.bid * BS + threadIdx.x); i < n; i += 2 * stride) {
         const int i2 = i + stride;

@@ -210,7 +210,8 @@ __device__ __forceinline__ bool reduce_last(const double (&loc)[K], double *part
 // post-smoothing pass with its two dots went from 21.8 to 19.8 us at 128^3 and
 // from 6.9 to 5.6 us on 128 x 128 x 1, the CG product at 128^3 from 19.3 to 17.8,
 // the update from 14.1 to 12.9; on eight columns the post-smoothing pass from
-// 121 to 104 us (one solve 1.02-1.14x by size).  The pair gains a
+// 121 to 104 us (times not overlapped by the kernels before; one solve
+// 1.02-1.14x by size).  The pair gains a
 // third word that takes the rounding errors of the second, so every addition
 // is error-free but for the last bits of the third word (TwoSum cascades as in
 // Ogita, Rump & Oishi 2005): about 70 bits, more than the FP64 tree kept.
